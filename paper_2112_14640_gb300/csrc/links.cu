@@ -7,8 +7,8 @@
 //    Grouping the paths by their last hop sigma gives the recursion
 //      W_s(n) = (1/k) sum_{mu: s_mu != 0} W_{s - s_mu mu}(n) V_{s_mu mu}(n + s - s_mu mu),
 //    evaluated level by level (k = 1..4) in shared memory, one thread block
-//    per site, in FP64 for FP64 operators and FP32 otherwise; the result is
-//    stored in the link precision;
+//    per tile of sites, in FP64 for FP64 operators and FP32 otherwise; the
+//    result is stored in the link precision;
 //  * build_clover: the clover term of Eq. (def_clov) in the block form of
 //    clover.cuh, from the clover-leaf field strength
 //      F_mu,nu(n) = (Q_mu,nu(n) - Q_mu,nu(n)^dag) / (8i),
@@ -17,6 +17,7 @@
 //  * stout_smear: the fat links V the paper builds its operators and F
 //    from (Sec. 2, App. F), steps of Morningstar-Peardon stout smearing.
 #include "bril_dirs.h"
+#include "hypercube.cuh"
 #include "internal.h"
 #include "linkalg.cuh"
 
@@ -67,91 +68,125 @@ __device__ __forceinline__ void signed_link(const UE *__restrict__ U, const Lat 
         }
 }
 
+// The caller's links [site][mu][a][b] with the boundary phase, in the
+// arithmetic type AB: the source of W for 16-bit link storage, whose own
+// links are already rounded (hyper::NativeLinks reads those of FP64 and FP32).
+template <int NC, typename UE, typename AB>
+struct CallerLinks {
+    const UE *U;
+    Lat g;
+    Phases ph;
+    __device__ __forceinline__ AB phase(long long site, int mu) const {
+        const Coord c = site_coords(g, site);
+        const int co = mu == 0 ? c.x : mu == 1 ? c.y : mu == 2 ? c.z : c.t;
+        const int ext = mu == 0 ? g.nx : mu == 1 ? g.ny : mu == 2 ? g.nz : g.nt;
+        const int bc = mu == 0 ? ph.bc[0] : mu == 1 ? ph.bc[1] : mu == 2 ? ph.bc[2] : ph.bc[3];
+        return co == ext - 1 ? (AB)bc : (AB)1;
+    }
+    __device__ __forceinline__ cx<AB> at(long long site, int mu, bool dag, int a, int b) const {
+        const cx<double> u = ld_u(U, (site * 4 + mu) * NC * NC + (dag ? b * NC + a : a * NC + b));
+        const AB f = phase(site, mu);   // +-1: exact after the conversion
+        return cx<AB>{f * (AB)u.re, f * (AB)(dag ? -u.im : u.im)};
+    }
+    __device__ __forceinline__ void load(long long site, int mu, bool dag, cx<AB> (&L)[NC][NC]) const {
+        const AB f = phase(site, mu);
+#pragma unroll
+        for (int a = 0; a < NC; ++a)
+#pragma unroll
+            for (int b = 0; b < NC; ++b) {
+                const cx<double> u = ld_u(U, (site * 4 + mu) * NC * NC + (dag ? b * NC + a : a * NC + b));
+                L[a][b] = cx<AB>{f * (AB)u.re, f * (AB)(dag ? -u.im : u.im)};
+            }
+    }
+};
+
 // W in FP64 for FP64 links, in FP32 otherwise (FP32 links carry 24 bits; the
 // four levels add a few FP32 roundings, and FP64 arithmetic is slow here).
-template <int NC, typename E>
+template <typename E>
 using WArith = std::conditional_t<sizeof(E) == 8, double, float>;
-// shared memory of build_w_kernel: the 81 W_s of one site
-template <int NC, typename E>
-constexpr size_t build_w_smem() { return sizeof(cx<WArith<NC, E>>) * 81 * NC * NC; }
 
-template <int NC, typename UE, typename E>
-__global__ void __launch_bounds__(96) build_w_kernel(const UE *__restrict__ U, E *__restrict__ W, Lat g, Phases ph) {
-    using AB = WArith<NC, E>;
-    // dynamic: 81 N_c^2 complex numbers exceed the static 48 KB for N_c >= 7 in FP64
+// The scale rho_k s_lead on a value of the builder's arithmetic type.  FP32:
+// the scale as a sum of two floats, so that the product carries one rounding
+// only, as it would from FP64, without the (slow) FP64 multiply.
+struct WScale {
+    float hi, lo;
+};
+__host__ __device__ constexpr WScale w_scale(double v) {
+    const float hi = (float)v;
+    return WScale{hi, (float)(v - (double)hi)};
+}
+__device__ __forceinline__ float scaled(float w, WScale s) { return __fmaf_rn(s.hi, w, __fmul_rn(s.lo, w)); }
+
+// store two consecutive complex numbers
+template <typename E, typename AB>
+__device__ __forceinline__ void store_pair(E *p, cx<AB> a, cx<AB> b) {
+    const cx<AB> v[2] = {a, b};
+    if constexpr (sizeof(E) <= 4) {
+        store_cx<E, 2, AB>(p, v);
+    } else {
+        store_cx<E, 1, AB>(p, v);
+        store_cx<E, 1, AB>(p + 2, v + 1);
+    }
+}
+
+// Level recursion W_s(n) = (1/k) sum_mu W_{s - s_mu mu}(n) V_{s_mu mu}(n + s - s_mu mu)
+// on a tile of S sites per block (hypercube.cuh).  Bound by the L1 / shared
+// memory pipe (216 products per site, each one link and one W operand) and by
+// writing W.  With one block per site and one thread per offset, every link
+// load touched as many cache lines as the warp has lanes and the FP64 phase
+// multiply and conversion of each element ran on the slow FP64 pipe: 4.96 ms
+// at 16^3x32, N_c = 3, FP32 from FP64 links, against 0.37 ms now (writing the
+// 755 MB of W takes 0.11 ms).  Lanes over consecutive sites make the link
+// loads contiguous, and the operator's own phased links need no conversion.
+template <int NC, typename E>
+struct WTile {
+    using AB = WArith<E>;
+    static constexpr int S = hyper::tile_sites(80, NC, sizeof(cx<AB>), true);
+    static constexpr int PAD = hyper::tile_pad(S);   // the transposed read of the output phase is conflict-free
+    static constexpr int R = 80 * NC * NC;           // rows of the tile: element e of W_q at q N_c^2 + e
+    static constexpr size_t smem = (size_t)R * PAD * sizeof(cx<AB>);
+};
+
+template <int NC, typename E, typename SRC>
+__global__ void __launch_bounds__(hyper::kThreads, 2) build_w_kernel(SRC src, E *__restrict__ W, Lat g) {
+    using AB = WArith<E>;
+    using T = WTile<NC, E>;
     extern __shared__ __align__(16) unsigned char w_smem[];
-    auto Ws = reinterpret_cast<cx<AB>(*)[NC * NC]>(w_smem);
-    const long long n = blockIdx.x;
-    const int dir = threadIdx.x < 81 ? kLevelOrder.d[threadIdx.x] : 81;   // offsets of a level share warps
-    const Coord c = site_coords(g, n);
-    const int x0[4] = {c.x, c.y, c.z, c.t};
-    const int ext[4] = {g.nx, g.ny, g.nz, g.nt};
-    int s[4] = {0, 0, 0, 0}, k = 0;
-    if (dir < 81) {
-        s[0] = dir % 3 - 1;
-        s[1] = (dir / 3) % 3 - 1;
-        s[2] = (dir / 9) % 3 - 1;
-        s[3] = dir / 27 - 1;
-        k = (s[0] != 0) + (s[1] != 0) + (s[2] != 0) + (s[3] != 0);
-        if (k == 0)
-            for (int a = 0; a < NC; ++a)
-                for (int b = 0; b < NC; ++b) Ws[40][a * NC + b] = cx<AB>{(AB)(a == b ? 1 : 0), (AB)0};
+    __shared__ WScale scale[80];
+    __shared__ double scale_d[sizeof(AB) == 8 ? 80 : 1];
+    cx<AB> *Ws = reinterpret_cast<cx<AB> *>(w_smem);
+    const long long n0 = (long long)blockIdx.x * T::S;
+    const int lane = threadIdx.x % T::S, worker = threadIdx.x / T::S;
+    // lanes past the last site repeat it; they store nothing below
+    const long long n = n0 + lane < g.V ? n0 + lane : g.V - 1;
+    const hyper::Steps st = hyper::steps_at(g, n);
+    if (threadIdx.x < 80) {
+        const hyper::Offset &o = hyper::kTable.o[threadIdx.x];
+        const double v = bril::rho(o.k) * (double)o.s[o.mu[o.k - 1]];   // the lead axis is the highest
+        scale[o.q] = w_scale(v);
+        if constexpr (sizeof(AB) == 8) scale_d[o.q] = v;
     }
-    const int pow3[4] = {1, 3, 9, 27};
-    // the last hop of the term along mu starts at n + s - s_mu mu
-    auto last_hop = [&](int mu, cx<AB> (&L)[NC][NC]) {
-        int m[4];
-        for (int nu = 0; nu < 4; ++nu) {
-            int v = x0[nu] + (nu == mu ? 0 : s[nu]);
-            m[nu] = (v + ext[nu]) % ext[nu];
-        }
-        signed_link<NC, UE, AB>(U, g, ph, m, mu, s[mu], L);
-    };
-    // N_c <= 4: every link this offset needs (one per axis it moves along) is
-    // requested before the first level, so that the four levels do not each
-    // wait for their own loads
-    constexpr bool kPreload = NC <= kMaxNcSmall;
-    cx<AB> Lpre[kPreload ? 4 : 1][NC][NC];   // by axis: compile-time indices keep them in registers
-    if constexpr (kPreload) {
-        if (dir < 81) {
+    constexpr int NW = hyper::kThreads / T::S;
+    auto row = [](int pos) { return (int)hyper::kTable.o[pos].q; };
+    hyper::w_level<1, NC, T::PAD, NW>(Ws, src, n, st, lane, worker, row);
+    hyper::w_level<2, NC, T::PAD, NW>(Ws, src, n, st, lane, worker, row);
+    hyper::w_level<3, NC, T::PAD, NW>(Ws, src, n, st, lane, worker, row);
+    hyper::w_level<4, NC, T::PAD, NW>(Ws, src, n, st, lane, worker, row);
+    // stored as rho_k s_lead W_s, [site][q][a][b] (bril_dirs.h): a site's rows
+    // are contiguous, two complex numbers per store (80 N_c^2 is even)
+    constexpr int H = T::R / 2;
+    for (int p = threadIdx.x; p < T::S * H; p += hyper::kThreads) {
+        const int site = p / H, r = 2 * (p - site * H);
+        if (n0 + site >= g.V) break;
+        cx<AB> v[2];
 #pragma unroll
-            for (int mu = 0; mu < 4; ++mu)
-                if (s[mu] != 0) last_hop(mu, Lpre[mu]);
+        for (int i = 0; i < 2; ++i) {
+            const cx<AB> w = Ws[(r + i) * T::PAD + site];
+            const int q = (r + i) / (NC * NC);
+            if constexpr (sizeof(AB) == 8) v[i] = scale_d[q] * w;
+            else v[i] = cx<AB>{scaled(w.re, scale[q]), scaled(w.im, scale[q])};
         }
-    }
-    __syncthreads();   // the identity at the centre feeds level 1
-    for (int level = 1; level <= 4; ++level) {
-        if (dir < 81 && k == level) {
-            cx<AB> acc[NC][NC];
-            for (int a = 0; a < NC; ++a)
-                for (int b = 0; b < NC; ++b) acc[a][b] = cx<AB>{0, 0};
-#pragma unroll
-            for (int mu = 0; mu < 4; ++mu) {
-                if (s[mu] == 0) continue;
-                const int prev = dir - s[mu] * pow3[mu];   // offset s - s_mu mu
-                cx<AB> Lrt[NC][NC];
-                if constexpr (!kPreload) last_hop(mu, Lrt);
-                const cx<AB>(&L)[NC][NC] = kPreload ? Lpre[kPreload ? mu : 0] : Lrt;
-                for (int a = 0; a < NC; ++a)
-                    for (int b = 0; b < NC; ++b)
-                        for (int q = 0; q < NC; ++q) cmac(acc[a][b], Ws[prev][a * NC + q], L[q][b]);
-            }
-            const AB inv = (AB)1 / (AB)level;
-            for (int a = 0; a < NC; ++a)
-                for (int b = 0; b < NC; ++b) Ws[dir][a * NC + b] = inv * acc[a][b];
-        }
-        __syncthreads();
-    }
-    if (dir < 81 && dir != 40) {
-        // stored as rho_k s_lead W_s at index q (bril_dirs.h)
-        double scale;
-        const int q = bril::store_index(s, &scale);
-        for (int e = 0; e < NC * NC; ++e) {
-            // [site][q][a][b] for either vector layout
-            const long long o = bril::w_index(q, e, n, NC);
-            W[2 * o] = from_acc<E, double>(scale * (double)Ws[dir][e].re);
-            W[2 * o + 1] = from_acc<E, double>(scale * (double)Ws[dir][e].im);
-        }
+        store_pair<E, AB>(W + 2 * ((n0 + site) * T::R + r), v[0], v[1]);
     }
 }
 
@@ -208,25 +243,35 @@ int launch_phase_links(dirac_op *op, const void *U, dirac_prec u_prec, cudaStrea
     });
 }
 
+template <int NC, typename E, typename SRC>
+static int run_build_w(const dirac_op *op, const SRC &src, cudaStream_t s) {
+    using T = WTile<NC, E>;
+    if constexpr (T::smem > 48 * 1024) {
+        const int rc = cuda_check(cudaFuncSetAttribute(build_w_kernel<NC, E, SRC>,
+                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem),
+                                  "build_w_kernel shared memory");
+        if (rc) return rc;
+    }
+    build_w_kernel<NC, E, SRC><<<grid_for(op->V, T::S), hyper::kThreads, T::smem, s>>>(src, (E *)op->w, op->lat);
+    return launch_check("build_w_kernel");
+}
+
+// W from the operator's phased links (already written by launch_phase_links on
+// the same stream) for FP64 and FP32 links, from the caller's field for 16-bit ones.
 int launch_build_w(dirac_op *op, const void *U, dirac_prec u_prec, cudaStream_t s) {
-    return dispatch_uprec(u_prec, [&](auto utag) {
-        using UE = std::remove_pointer_t<decltype(utag)>;
-        return dispatch_prec(link_prec(op), [&](auto tag) {
-            using E = std::remove_pointer_t<decltype(tag)>;
-            return dispatch_nc<big_nc_ok<E>()>(op->nc, [&](auto ncc) {
-                constexpr int NC = decltype(ncc)::value;
-                constexpr size_t smem = build_w_smem<NC, E>();
-                if constexpr (smem > 48 * 1024) {
-                    const int rc = cuda_check(cudaFuncSetAttribute(build_w_kernel<NC, UE, E>,
-                                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                                   (int)smem),
-                                              "build_w_kernel shared memory");
-                    if (rc) return rc;
-                }
-                build_w_kernel<NC, UE, E><<<(unsigned)op->V, 96, smem, s>>>((const UE *)U, (E *)op->w, op->lat,
-                                                                          phases_of(op));
-                return launch_check("build_w_kernel");
-            });
+    return dispatch_prec(link_prec(op), [&](auto tag) {
+        using E = std::remove_pointer_t<decltype(tag)>;
+        return dispatch_nc<big_nc_ok<E>()>(op->nc, [&](auto ncc) {
+            constexpr int NC = decltype(ncc)::value;
+            if constexpr (sizeof(E) >= 4) {
+                return run_build_w<NC, E>(op, hyper::NativeLinks<NC, E, WArith<E>>{(const E *)op->links}, s);
+            } else {
+                return dispatch_uprec(u_prec, [&](auto utag) {
+                    using UE = std::remove_pointer_t<decltype(utag)>;
+                    return run_build_w<NC, E>(
+                        op, CallerLinks<NC, UE, WArith<E>>{(const UE *)U, op->lat, phases_of(op)}, s);
+                });
+            }
         });
     });
 }
