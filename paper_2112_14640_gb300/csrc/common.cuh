@@ -59,6 +59,78 @@ __device__ __forceinline__ void rmac(cx<A> &acc, A s, cx<A> a) {
     acc.im = fma(s, a.im, acc.im);
 }
 
+// --------------------------------------------------- packed FP32 arithmetic
+// Two FP32 multiply-adds per instruction (fma.rn.f32x2): the FP32 pipe takes
+// as long as for two scalar ones, but one issue slot instead of two, which is
+// what bounds a stencil whose products dominate.  A complex number is the pair
+// (re, im) as it is stored, so a product w f with w = (re, im) splits into
+// re f and im f with re and im broadcast, and a sum of products needs no
+// swapped copies of f: Prod::Acc keeps sum(re f) and sum(im f) apart, and the
+// value is sum(re f) + i sum(im f).
+struct pk2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ pk2 pack2(float a, float b) {
+    pk2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ pk2 bcast2(float a) { return pack2(a, a); }
+__device__ __forceinline__ cx<float> unpack2(pk2 a) {
+    cx<float> r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.re), "=f"(r.im) : "l"(a.v));
+    return r;
+}
+__device__ __forceinline__ pk2 fma2(pk2 a, pk2 b, pk2 c) {
+    pk2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return d;
+}
+__device__ __forceinline__ pk2 mul2(pk2 a, pk2 b) {
+    pk2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d.v) : "l"(a.v), "l"(b.v));
+    return d;
+}
+
+// A vector component, a matrix element as a multiplier, and an accumulator of
+// products: plain complex arithmetic, or packed (FP32).
+template <typename A, bool PACK>
+struct Prod {
+    using Vec = cx<A>;
+    struct Mul {
+        cx<A> w;
+    };
+    struct Acc {
+        cx<A> s = {0, 0};
+        __device__ __forceinline__ void mac(const Mul &w, const Vec &f) { cmac(s, w.w, f); }
+        __device__ __forceinline__ cx<A> value() const { return s; }
+    };
+    static __device__ __forceinline__ Vec vec(cx<A> a) { return a; }
+    static __device__ __forceinline__ Mul mul(cx<A> a) { return Mul{a}; }
+    static __device__ __forceinline__ Vec scale(A f, const Vec &v) { return f * v; }
+};
+template <>
+struct Prod<float, true> {
+    using Vec = pk2;
+    struct Mul {
+        pk2 re, im;
+    };
+    struct Acc {
+        pk2 r = {0}, i = {0};
+        __device__ __forceinline__ void mac(const Mul &w, const Vec &f) {
+            r = fma2(w.re, f, r);
+            i = fma2(w.im, f, i);
+        }
+        __device__ __forceinline__ cx<float> value() const {
+            const cx<float> a = unpack2(r), b = unpack2(i);
+            return cx<float>{a.re - b.im, a.im + b.re};
+        }
+    };
+    static __device__ __forceinline__ Vec vec(cx<float> a) { return pack2(a.re, a.im); }
+    static __device__ __forceinline__ Mul mul(cx<float> a) { return Mul{bcast2(a.re), bcast2(a.im)}; }
+    static __device__ __forceinline__ Vec scale(float f, const Vec &v) { return mul2(bcast2(f), v); }
+};
+
 // -------------------------------------------------------- storage elements
 template <typename E> struct Acc { using T = float; };
 template <> struct Acc<double> { using T = double; };

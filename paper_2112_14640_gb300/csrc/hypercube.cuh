@@ -44,25 +44,21 @@ __host__ __device__ constexpr Table make_table() {
     const int pow3[4] = {1, 3, 9, 27};
     int i = 0;
     t.pos[40] = -1;
-    for (int k = 1; k <= 4; ++k) {
-        int q = 0;
-        for (int m = 1; m < 16; ++m)
-            for (int b = 0; b < (1 << bril::popc4(m)); ++b, ++q) {
-                if (bril::popc4(m) != k) continue;
-                Offset &o = t.o[i];
-                int j = 0;
-                for (int mu = 0; mu < 4; ++mu) {
-                    o.s[mu] = 0;
-                    if ((m >> mu) & 1) {
-                        o.s[mu] = ((b >> j) & 1) ? -1 : 1;
-                        o.mu[j++] = (unsigned char)mu;
-                    }
-                }
-                o.k = (unsigned char)k;
-                o.q = (unsigned char)q;
-                t.pos[dir_index(o.s)] = i++;
+    for (int k = 1; k <= 4; ++k)
+        for (int d = 0; d < 81; ++d) {
+            const int s[4] = {d % 3 - 1, (d / 3) % 3 - 1, (d / 9) % 3 - 1, d / 27 - 1};
+            if ((s[0] != 0) + (s[1] != 0) + (s[2] != 0) + (s[3] != 0) != k) continue;
+            Offset &o = t.o[i];
+            int j = 0;
+            for (int mu = 0; mu < 4; ++mu) {
+                o.s[mu] = (signed char)s[mu];
+                if (s[mu]) o.mu[j++] = (unsigned char)mu;
             }
-    }
+            double scale = 0;
+            o.k = (unsigned char)k;
+            o.q = (unsigned char)bril::store_index(s, &scale);
+            t.pos[d] = i++;
+        }
     for (i = 0; i < 80; ++i) {
         Offset &o = t.o[i];
         const int d = dir_index(o.s);

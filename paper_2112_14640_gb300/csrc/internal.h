@@ -95,6 +95,16 @@ int dispatch_prec(dirac_prec p, F &&f) {
 // per thread and the compiler's own register choice (kMaxNcSmall below).
 constexpr int kMaxNc = 8;
 constexpr int kMaxNcSmall = 4;
+// Products of a stencil over the Brillouin offsets: packed FP32 pairs
+// (common.cuh) where the two accumulators of each of the NC NS VR components
+// leave the register class (the cap of MINB, below) about 60
+// registers for the rest; plain ones where they would spill, and above N_c = 4.
+template <int NC, int NS, int VR, int MINB>
+constexpr bool packed_fits() {
+    return NC <= kMaxNcSmall && 4 * NC * NS * VR + 60 <= (MINB > 1 ? 65536 / (128 * MINB) : 208);
+}
+template <int NC, int NS, int VR, int MINB, typename A>
+using StencilProd = Prod<A, sizeof(A) == 4 && packed_fits<NC, NS, VR, MINB>()>;
 template <bool BIG = true, typename F>
 int dispatch_nc(int nc, F &&f) {
     switch (nc) {
@@ -205,10 +215,15 @@ inline void launch_variant(const dirac_op *op, int &vr, int &minb, int &block) {
             minb = vr == 4 ? 3 : 4;
         } else if (op->kind == DIRAC_STAGGERED) {
             minb = 3;
-        } else if (op->kind == DIRAC_BRILLOUIN && vr <= 2) {
-            minb = 3;
-            block = 384;
         }
+    }
+    // 81-point stencils on 4 spins in FP32 arithmetic: two accumulators per
+    // component (common.cuh), so one RHS per thread from N_c = 3 on (16^3x32,
+    // N_v = 12, D_B: 1.07 ms, two RHS 1.06 ms at 8 warps per SM; the Brillouin
+    // Laplacian 0.94 against 1.13 ms)
+    if (uses_w(op->kind) && spins_of(op->kind) == 4 && op->prec != DIRAC_F64 && op->nc <= kMaxNcSmall) {
+        vr = op->nc >= 3 || vr == 1 ? 1 : 2;
+        if (op->nc == 3) minb = 4;
     }
 }
 

@@ -11,10 +11,14 @@
 // Laplacian reads the operator's stored W~_q = rho_k s_lead W_s (bril_dirs.h),
 // per site in visiting order, and weighs each with -c_k s_lead, which is
 // -lambda_k/2 on W_s; offsets and weights come from a table in constant
-// memory (one broadcast read per offset, uniform over the warp).
+// memory (one broadcast read per offset, uniform over the warp).  W~ is staged
+// in shared memory for the block (wstage.cuh) and its products are packed
+// (common.cuh): blap 0.991 -> 0.946 ms, bsuv 0.490 -> 0.313 ms at 16^3x32,
+// N_v = 12, N_c = 3, FP32.
 #pragma once
 #include "bril_dirs.h"
 #include "internal.h"
+#include "wstage.cuh"
 
 namespace dgb {
 namespace bril {
@@ -27,20 +31,14 @@ struct OffsetTable {
 };
 __host__ __device__ constexpr OffsetTable make_offset_table() {
     OffsetTable t{};
-    int q = 0;
-    for (int m = 1; m < 16; ++m) {
-        const int k = popc4(m);
-        for (int b = 0; b < (1 << k); ++b, ++q) {
-            int j = 0;
-            for (int mu = 0; mu < 4; ++mu) {
-                t.s[q][mu] = 0;
-                if ((m >> mu) & 1) {
-                    t.s[q][mu] = ((b >> j) & 1) ? -1 : 1;
-                    ++j;
-                }
-            }
-            t.lap[q] = -c_lambda(k) * (double)t.s[q][lead_axis(m)];
-        }
+    for (int d = 0; d < 81; ++d) {
+        const int s[4] = {d % 3 - 1, (d / 3) % 3 - 1, (d / 9) % 3 - 1, d / 27 - 1};
+        const int k = (s[0] != 0) + (s[1] != 0) + (s[2] != 0) + (s[3] != 0);
+        if (k == 0) continue;
+        double scale = 0;
+        const int q = store_index(s, &scale);
+        for (int mu = 0; mu < 4; ++mu) t.s[q][mu] = (signed char)s[mu];
+        t.lap[q] = -c_lambda(k) * (scale < 0 ? -1.0 : 1.0);
     }
     return t;
 }
@@ -49,65 +47,43 @@ __host__ __device__ constexpr OffsetTable make_offset_table() {
 
 static __constant__ bril::OffsetTable kLapOffsets = bril::make_offset_table();
 
-// Whether a hop multiplies its weight into the N_c x N_c matrix once (N_c^2
-// complex scalings) instead of into each of the NS VR N_c products (one real
-// multiply-add per complex component): worth it when NS VR > N_c.
+// Whether a hop multiplies its weight into the N_c x N_c matrix (N_c^2 complex
+// scalings) or into the NS VR N_c vector components it reads.
 template <int NC, int NS, int VR>
 constexpr bool fold_weight() { return NS * VR > NC; }
 
 // acc[c][s] += f L psi(m) (or f L^dag psi(m)) for every spin component s
-template <int NC, int NS, int VR, bool DAG, typename E, typename A>
-__device__ __forceinline__ void lap_hop(cx<A> (&acc)[NC][NS][VR], const cx<A> (&Lin)[NC][NC],
+template <typename P, int NC, int NS, int VR, bool DAG, typename E, typename A>
+__device__ __forceinline__ void lap_hop(typename P::Acc (&acc)[NC][NS][VR], const cx<A> (&L)[NC][NC],
                                         const E *__restrict__ psi, long long cs_stride, A f) {
     constexpr bool FOLD = fold_weight<NC, NS, VR>();
-    cx<A> Lf[NC][NC];
-    if constexpr (FOLD) {
+    // one colour component of the neighbour at a time: column k of the matrix
+    // and NS VR vector components in registers
 #pragma unroll
-        for (int a = 0; a < NC; ++a)
+    for (int k = 0; k < NC; ++k) {
+        typename P::Mul w[NC];
 #pragma unroll
-            for (int b = 0; b < NC; ++b) Lf[a][b] = cx<A>{f * Lin[a][b].re, f * Lin[a][b].im};
-    }
-    const cx<A>(*L)[NC] = FOLD ? (const cx<A>(*)[NC])Lf : Lin;
+        for (int c = 0; c < NC; ++c) {
+            const cx<A> u = DAG ? conj(L[k][c]) : L[c][k];
+            w[c] = P::mul(FOLD ? f * u : u);
+        }
 #pragma unroll
-    for (int s = 0; s < NS; ++s) {
-        if constexpr (FOLD) {
-            // one colour component of the neighbour at a time (VR complex
-            // numbers in registers, not N_c VR)
+        for (int s = 0; s < NS; ++s) {
+            cx<A> p[VR];
+            load_cx<E, VR, A>(psi + 2 * (k * NS + s) * cs_stride, p);
 #pragma unroll
-            for (int k = 0; k < NC; ++k) {
-                cx<A> pk[VR];
-                load_cx<E, VR, A>(psi + 2 * (k * NS + s) * cs_stride, pk);
+            for (int v = 0; v < VR; ++v) {
+                const typename P::Vec pv = FOLD ? P::vec(p[v]) : P::scale(f, P::vec(p[v]));
 #pragma unroll
-                for (int c = 0; c < NC; ++c)
-#pragma unroll
-                    for (int v = 0; v < VR; ++v) {
-                        if constexpr (DAG) cmac_conj(acc[c][s][v], L[k][c], pk[v]);
-                        else cmac(acc[c][s][v], L[c][k], pk[v]);
-                    }
+                for (int c = 0; c < NC; ++c) acc[c][s][v].mac(w[c], pv);
             }
-        } else {
-            cx<A> p[NC][VR];
-#pragma unroll
-            for (int k = 0; k < NC; ++k) load_cx<E, VR, A>(psi + 2 * (k * NS + s) * cs_stride, p[k]);
-#pragma unroll
-            for (int c = 0; c < NC; ++c)
-#pragma unroll
-                for (int v = 0; v < VR; ++v) {
-                    cx<A> t = {0, 0};
-#pragma unroll
-                    for (int k = 0; k < NC; ++k) {
-                        if constexpr (DAG) cmac_conj(t, L[k][c], p[k][v]);
-                        else cmac(t, L[c][k], p[k][v]);
-                    }
-                    rmac(acc[c][s][v], f, t);
-                }
         }
     }
 }
 
-template <int NC, int NS, int VR, int LAYOUT, typename E, typename A>
+template <typename P, int NC, int NS, int VR, int LAYOUT, typename E, typename A>
 __device__ __forceinline__ void lap_write(const E *__restrict__ in, E *__restrict__ out, const Lat &g,
-                                          long long n, int j, A centre, const cx<A> (&acc)[NC][NS][VR]) {
+                                          long long n, int j, A centre, const typename P::Acc (&acc)[NC][NS][VR]) {
     using L = Layout<LAYOUT>;
     const long long cs = L::cs_stride(g);
     const long long base = 2 * (L::vec(g, n, NC * NS, 0) + (long long)j * VR);
@@ -119,7 +95,7 @@ __device__ __forceinline__ void lap_write(const E *__restrict__ in, E *__restric
             const long long off = base + 2LL * (a * NS + s) * cs;
             load_cx<E, VR, A>(in + off, p);
 #pragma unroll
-            for (int v = 0; v < VR; ++v) o[v] = centre * p[v] + acc[a][s][v];
+            for (int v = 0; v < VR; ++v) o[v] = centre * p[v] + acc[a][s][v].value();
             store_cx<E, VR, A>(out + off, o);
         }
 }
@@ -141,13 +117,9 @@ __global__ void __launch_bounds__(stencil_max_threads(MINB), (MINB > 1 ? 1 : 0))
     const Coord c = site_coords(g, n);
     const long long cs = L::cs_stride(g), ls = L::template mat_stride<NC>(g);
 
-    cx<A> acc[NC][NS][VR];
-#pragma unroll
-    for (int a = 0; a < NC; ++a)
-#pragma unroll
-        for (int s = 0; s < NS; ++s)
-#pragma unroll
-            for (int v = 0; v < VR; ++v) acc[a][s][v] = cx<A>{0, 0};
+    using P = Prod<A, false>;   // packed products measured slower here (0.121 vs 0.115 ms): the second
+                                // accumulator costs warps, and the loads bound this kernel
+    typename P::Acc acc[NC][NS][VR];
     const A mhalf = (A)-0.5;
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
@@ -155,23 +127,31 @@ __global__ void __launch_bounds__(stencil_max_threads(MINB), (MINB > 1 ? 1 : 0))
         const long long bw = neighbour(g, n, c, mu, -1);
         cx<A> Lm[NC][NC];
         load_mat_s<NC, E, A>(U + 2 * L::template mat<NC>(g, n, 4, mu), ls, Lm);
-        lap_hop<NC, NS, VR, false>(acc, Lm, in + 2 * (L::vec(g, fw, NC * NS, 0) + (long long)j * VR), cs, mhalf);
+        lap_hop<P, NC, NS, VR, false, E, A>(acc, Lm, in + 2 * (L::vec(g, fw, NC * NS, 0) + (long long)j * VR), cs, mhalf);
         load_mat_s<NC, E, A>(U + 2 * L::template mat<NC>(g, bw, 4, mu), ls, Lm);
-        lap_hop<NC, NS, VR, true>(acc, Lm, in + 2 * (L::vec(g, bw, NC * NS, 0) + (long long)j * VR), cs, mhalf);
+        lap_hop<P, NC, NS, VR, true, E, A>(acc, Lm, in + 2 * (L::vec(g, bw, NC * NS, 0) + (long long)j * VR), cs, mhalf);
     }
-    lap_write<NC, NS, VR, LAYOUT, E, A>(in, out, g, n, j, centre, acc);
+    lap_write<P, NC, NS, VR, LAYOUT, E, A>(in, out, g, n, j, centre, acc);
 }
 
 // Eq. (app_blap): centre = m^2/2 - lambda_0/2, offset q weighted kLapOffsets.lap[q] on W~_q
-template <int NC, int NS, int VR, typename E, int MINB, int LAYOUT>
+// STAGED: W~ through shared memory, one ring per block (wstage.cuh); else each
+// thread reads its own.
+template <int NC, int NS, int VR, typename E, int MINB, int LAYOUT, bool STAGED>
 __global__ void __launch_bounds__(stencil_max_threads(MINB), (MINB > 1 ? 1 : 0))
     blap_kernel(const E *__restrict__ W, const E *__restrict__ in, E *__restrict__ out, Lat g,
                 typename Acc<E>::T centre) {
     using A = typename Acc<E>::T;
     using L = Layout<LAYOUT>;
     const int nchunk = g.nv / VR;
-    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (tid >= g.nsites * nchunk) return;
+    const long long total = g.nsites * nchunk, tid0 = (long long)blockIdx.x * blockDim.x;
+    long long tid = tid0 + threadIdx.x;
+    // a staged block's threads all copy and wait; those past the end repeat the last one's work
+    const bool live = tid < total;
+    if (!live) {
+        if constexpr (!STAGED) return;
+        tid = total - 1;
+    }
     long long i;
     int j;
     split_tid(tid, nchunk, i, j);
@@ -192,15 +172,9 @@ __global__ void __launch_bounds__(stencil_max_threads(MINB), (MINB > 1 ? 1 : 0))
             stride *= ext[mu];
         }
     }
-    cx<A> acc[NC][NS][VR];
-#pragma unroll
-    for (int a = 0; a < NC; ++a)
-#pragma unroll
-        for (int s = 0; s < NS; ++s)
-#pragma unroll
-            for (int v = 0; v < VR; ++v) acc[a][s][v] = cx<A>{0, 0};
+    using P = StencilProd<NC, NS, VR, MINB, A>;
+    typename P::Acc acc[NC][NS][VR];
     // W~ of one site contiguous in visiting order (either vector layout)
-    const E *wp = W + 2LL * n * 80 * NC * NC;
     const E *inj = in + 2LL * j * VR;
     auto hop = [&](int q, const cx<A>(&Wm)[NC][NC]) {
         int m = (int)n;
@@ -209,10 +183,36 @@ __global__ void __launch_bounds__(stencil_max_threads(MINB), (MINB > 1 ? 1 : 0))
             const int sm = kLapOffsets.s[q][mu];
             m += sm > 0 ? dp[mu] : (sm < 0 ? dm[mu] : 0);
         }
-        lap_hop<NC, NS, VR, false>(acc, Wm, inj + 2 * L::vec(g, (long long)m, NC * NS, 0), cs,
-                                   (A)kLapOffsets.lap[q]);
+        lap_hop<P, NC, NS, VR, false, E, A>(acc, Wm, inj + 2 * L::vec(g, (long long)m, NC * NS, 0), cs,
+                                         (A)kLapOffsets.lap[q]);
     };
-    if constexpr (NC <= kMaxNcSmall) {
+    if constexpr (STAGED) {
+        extern __shared__ __align__(16) unsigned char w_ring[];
+        const long long s0 = tid0 / nchunk, end = tid0 + blockDim.x < total ? tid0 + blockDim.x : total;
+        wst::Ring<NC, E> ring;
+        ring.src = reinterpret_cast<const unsigned char *>(W + 2LL * (g.n0 + s0) * 80 * NC * NC);
+        ring.smem = w_ring;
+        ring.nsites = (int)((end - 1) / nchunk - s0 + 1);
+        ring.slots = wst::block_sites(blockDim.x, nchunk);
+        ring.mine = (int)(i - s0);
+        ring.start();
+        int q = 0;
+#pragma unroll 1
+        for (int stage = 0; stage < wst::kStages; ++stage) {
+            const E *w = ring.enter(stage);
+            const int end_q = 2 + 6 * stage;
+#pragma unroll 1
+            for (; q < end_q; q += 2, w += 4 * NC * NC) {
+                cx<A> Wm[NC][NC];
+                wst::load_mat_shared<NC, E, A>(w, Wm);
+                hop(q, Wm);
+                wst::load_mat_shared<NC, E, A>(w + 2 * NC * NC, Wm);
+                hop(q + 1, Wm);
+            }
+        }
+        if (!live) return;
+    } else if constexpr (NC <= kMaxNcSmall) {
+        const E *wp = W + 2LL * n * 80 * NC * NC;
         // two offsets per trip: the W~ of the next offset is loaded while the
         // current one is applied, the two buffers swapping roles (80 is even)
         cx<A> Wa[NC][NC], Wb[NC][NC];
@@ -225,6 +225,7 @@ __global__ void __launch_bounds__(stencil_max_threads(MINB), (MINB > 1 ? 1 : 0))
             hop(q + 1, Wb);
         }
     } else {
+        const E *wp = W + 2LL * n * 80 * NC * NC;
         // large N_c: one N_c x N_c buffer (the register file holds no second one)
 #pragma unroll 1
         for (int q = 0; q < 80; ++q) {
@@ -233,7 +234,7 @@ __global__ void __launch_bounds__(stencil_max_threads(MINB), (MINB > 1 ? 1 : 0))
             hop(q, Wm);
         }
     }
-    lap_write<NC, NS, VR, LAYOUT, E, A>(in, out, g, n, j, centre, acc);
+    lap_write<P, NC, NS, VR, LAYOUT, E, A>(in, out, g, n, j, centre, acc);
 }
 
 template <typename E, int LAYOUT>
@@ -248,22 +249,53 @@ int launch_laplace_v(const dirac_op *op, const void *in, void *out, double m, cu
         return dispatch_vr(vr, [&](auto vrc) {
             constexpr int VR = decltype(vrc)::value;
             if constexpr (!vr_compiled<NC>(VR)) return (int)DIRAC_ERR_INVALID_ARG;
-            else return dispatch_minb<NC>(minb, [&](auto mbc) {
-                constexpr int MINB = decltype(mbc)::value;
-                const long long threads = op->lat.nsites * (op->nv / VR);
-                auto go = [&](auto nsc) {
-                    constexpr int NS = decltype(nsc)::value;
-                    if (bril)
-                        blap_kernel<NC, NS, VR, E, MINB, LAYOUT><<<grid_for(threads, block), block, 0, s>>>(
-                            (const E *)op->w, (const E *)in, (E *)out, op->lat, (A)centre);
-                    else
-                        wlap_kernel<NC, NS, VR, E, MINB, LAYOUT><<<grid_for(threads, block), block, 0, s>>>(
-                            (const E *)op->links, (const E *)in, (E *)out, op->lat, (A)centre);
-                    return launch_check(bril ? "blap_kernel" : "wlap_kernel");
+            else {
+                const int nchunk = op->nv / VR;
+                const long long threads = op->lat.nsites * nchunk;
+                auto on_spins = [&](auto &&go) {
+                    return spins_of(op->kind) == 4 ? go(std::integral_constant<int, 4>{})
+                                                   : go(std::integral_constant<int, 1>{});
                 };
-                return spins_of(op->kind) == 4 ? go(std::integral_constant<int, 4>{})
-                                               : go(std::integral_constant<int, 1>{});
-            });
+                auto run_w = [&](auto kernel, int T, size_t smem) {
+                    if (smem > 48 * 1024) {
+                        const int rc = cuda_check(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                                       (int)wst::kMaxSmem),
+                                                  "blap_kernel shared memory");
+                        if (rc) return rc;
+                    }
+                    kernel<<<grid_for(threads, T), T, smem, s>>>((const E *)op->w, (const E *)in, (E *)out, op->lat,
+                                                                (A)centre);
+                    return launch_check("blap_kernel");
+                };
+                if (!bril)
+                    return dispatch_minb<NC>(minb, [&](auto mbc) {
+                        constexpr int MINB = decltype(mbc)::value;
+                        return on_spins([&](auto nsc) {
+                            constexpr int NS = decltype(nsc)::value;
+                            wlap_kernel<NC, NS, VR, E, MINB, LAYOUT><<<grid_for(threads, block), block, 0, s>>>(
+                                (const E *)op->links, (const E *)in, (E *)out, op->lat, (A)centre);
+                            return launch_check("wlap_kernel");
+                        });
+                    });
+                const size_t smem = NC <= kMaxNcSmall ? wst::smem_bytes<NC, E>(block, nchunk) : 0;
+                if (NC > kMaxNcSmall || nchunk < wst::kMinChunks || smem > wst::kMaxSmem)
+                    // few threads share a site's W~
+                    return on_spins([&](auto nsc) {
+                        constexpr int NS = decltype(nsc)::value;
+                        return run_w(blap_kernel<NC, NS, VR, E, 1, LAYOUT, false>,
+                                     block <= kStencilBlock ? block : kStencilBlock, 0);
+                    });
+                if constexpr (NC <= kMaxNcSmall) {
+                    return dispatch_minb<NC>(minb, [&](auto mbc) {
+                        constexpr int MINB = decltype(mbc)::value;
+                        return on_spins([&](auto nsc) {
+                            constexpr int NS = decltype(nsc)::value;
+                            return run_w(blap_kernel<NC, NS, VR, E, MINB, LAYOUT, true>, block, smem);
+                        });
+                    });
+                }
+                return (int)DIRAC_ERR_INVALID_ARG;
+            }
         });
     });
 }
