@@ -278,8 +278,9 @@ int dirac_op_get_launch(const dirac_op *op, int *vr, int *minb, int *block);
 /* Time every compiled variant of D (bare mass m0) on operator-owned buffers
  * and keep the fastest for this operator; the choice is also remembered for
  * operators created later in this process with the same kind, layout,
- * precision, link storage, N_c, N_v and volume (including the
- * lower-precision twins of mixed solves).
+ * precision, link storage, N_c, N_v and volume (including what the solvers
+ * iterate with: the site-inner form of the operator, and the site-inner
+ * lower-precision twin of a mixed solve).
  * best_ms (may be NULL) receives the winner's time per apply.  Synchronises. */
 int dirac_op_autotune(dirac_op *op, double m0, void *stream, double *best_ms);
 
@@ -401,8 +402,11 @@ typedef struct {
 } dirac_solve_stats;
 
 /* Solve for N_v right-hand sides b (operator precision); x holds the initial
- * guess on entry and the solution on exit.  Blocks until done (it reads
- * per-iteration residual norms on the host).  stats may be NULL. */
+ * guess on entry and the solution on exit.  The iteration runs on site-inner
+ * vectors whatever the operator's layout (b and x of a site-outer operator are
+ * reordered inside).  Blocks until done (CG reads the residual norms of a run
+ * of iterations on the host at the run's end, BiCGstab those of each
+ * iteration).  stats may be NULL. */
 int dirac_solve(const dirac_op *op, const void *b, void *x, double m0,
                 const dirac_solve_params *params, dirac_solve_stats *stats, void *stream);
 

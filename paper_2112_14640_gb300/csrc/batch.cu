@@ -25,9 +25,6 @@
 
 namespace dgb {
 
-int solver_ws(const dirac_op *op, void **vecs, int nvecs, double **scal);
-int batch_apply_A_pq(const dirac_op *op, const void *p, void *q, double *pq, double m0, cudaStream_t s);
-
 __device__ __forceinline__ unsigned long long globaltimer() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -36,25 +33,6 @@ __device__ __forceinline__ unsigned long long globaltimer() {
 
 __global__ void stamp_kernel(unsigned long long *t) {
     if (threadIdx.x == 0 && blockIdx.x == 0) *t = globaltimer();
-}
-
-// pq holds N_v real values |D p|^2
-__global__ void batch_alpha_kernel(int nv, const double *rr, const double *pq, const double *act, double *alpha) {
-    const int v = threadIdx.x;
-    if (v >= nv) return;
-    const double p = pq[v];
-    const double a = (act[v] != 0.0 && p > 0.0) ? rr[v] / p : 0.0;
-    alpha[2 * v] = a;
-    alpha[2 * v + 1] = 0.0;
-}
-
-__global__ void batch_beta_kernel(int nv, const double *rr_new, double *rr, const double *act, double *beta) {
-    const int v = threadIdx.x;
-    if (v >= nv) return;
-    const double b = (act[v] != 0.0 && rr[v] > 0.0) ? rr_new[v] / rr[v] : 0.0;
-    beta[2 * v] = b;
-    beta[2 * v + 1] = 0.0;
-    rr[v] = rr_new[v];
 }
 
 // After a recompute: freeze the RHS whose true residual passes; when all have
@@ -144,23 +122,32 @@ extern "C" int dirac_solve_batched(int nsolves, dirac_op *const *ops, const void
     unsigned long long *dstart = nullptr;
     std::vector<BatchState> hstate(nsolves);
     unsigned long long hstart = 0;
+    // each solve iterates on site-inner vectors: the view it applies and, for a
+    // site-outer operator, a reordered solution (vec 4)
+    std::vector<dirac_op> views(nsolves);
+    std::vector<void *> xi(nsolves);
     std::vector<void *> vecs(nsolves * 4);
-    std::vector<double *> scal(nsolves);
+    std::vector<CgScalars> scal(nsolves);   // no stop rule: the segment's check decides
     int rc = DIRAC_OK, replays = 0;
     const int max_replays = (prm->maxit + K - 1) / K;
     auto t0 = std::chrono::steady_clock::now();
 
-    // per solve: rhs (vec 3), r (0), p (1), q (2); scalars: rr, rr_new, pq, alpha, beta, act, nb
+    // per solve: rhs (vec 3), r (0), p (1), q (2), and the CG scalars
     TRYB(cuda_check(cudaStreamCreateWithFlags(&main, cudaStreamNonBlocking), "stream"));
     TRYB(cuda_check(cudaEventCreateWithFlags(&entry, cudaEventDisableTiming), "event"));
     TRYB(cuda_check(cudaEventRecord(entry, user), "entry"));
     TRYB(cuda_check(cudaStreamWaitEvent(main, entry, 0), "wait entry"));
     for (int i = 0; i < nsolves; ++i) {
-        void *v4[4];
-        double *sc = nullptr;
-        TRYB(solver_ws(ops[i], v4, 4, &sc));
-        for (int k = 0; k < 4; ++k) vecs[i * 4 + k] = v4[k];
-        scal[i] = sc;
+        void *ws[5];
+        TRYB(solver_cg(ops[i], ws, 5, &scal[i], main));
+        for (int k = 0; k < 4; ++k) vecs[i * 4 + k] = ws[k];
+        views[i] = op_site_inner(ops[i]);
+        xi[i] = x[i];
+        if (ops[i]->geom.layout != DIRAC_LAYOUT_SITE_INNER) {
+            xi[i] = ws[4];
+            TRYB(blas_convert_layout(ops[i], x[i], ops[i]->prec, ops[i]->geom.layout, xi[i], ops[i]->prec,
+                                     DIRAC_LAYOUT_SITE_INNER, main));
+        }
     }
     TRYB(cuda_check(cudaMalloc(&dstate, nsolves * sizeof(BatchState)), "batch state"));
     TRYB(cuda_check(cudaMalloc(&dstart, sizeof(unsigned long long)), "batch stamp"));
@@ -173,16 +160,20 @@ extern "C" int dirac_solve_batched(int nsolves, dirac_op *const *ops, const void
     stamp_kernel<<<1, 1, 0, main>>>(dstart);
     // set-up on the main stream: rhs, r = rhs - A x, p = r, norms, masks
     for (int i = 0; i < nsolves; ++i) {
-        const dirac_op *op = ops[i];
+        const dirac_op *op = &views[i];
         const dirac_prec p = op->prec;
         const int nv = op->nv;
         void *r = vecs[i * 4 + 0], *pv = vecs[i * 4 + 1], *q = vecs[i * 4 + 2], *rhs = vecs[i * 4 + 3];
-        double *sc = scal[i];
-        double *rr = sc, *nb = sc + 6 * 128, *act = sc + 5 * 128;
-        if (prm->solver == DIRAC_CG_NORMAL) TRYB(op_apply(op, b[i], rhs, m0[i], -1, main));
-        else TRYB(blas_axpby(op, p, rhs, b[i], nullptr, 1.0, nullptr, nullptr, 0.0, nullptr, main));
+        const void *bi = b[i];
+        if (ops[i]->geom.layout != DIRAC_LAYOUT_SITE_INNER) {
+            TRYB(blas_convert_layout(ops[i], b[i], p, ops[i]->geom.layout, pv, p, DIRAC_LAYOUT_SITE_INNER, main));
+            bi = pv;
+        }
+        double *rr = scal[i].rr, *nb = const_cast<double *>(scal[i].nb), *act = const_cast<double *>(scal[i].act);
+        if (prm->solver == DIRAC_CG_NORMAL) TRYB(op_apply(op, bi, rhs, m0[i], -1, main));
+        else TRYB(blas_axpby(op, p, rhs, bi, nullptr, 1.0, nullptr, nullptr, 0.0, nullptr, main));
         TRYB(blas_norm2(op, p, rhs, nb, main));
-        TRYB(op_apply_cg(op, x[i], q, m0[i], main));
+        TRYB(op_apply_cg(op, xi[i], q, m0[i], main));
         TRYB(blas_axpby(op, p, r, rhs, nullptr, 1.0, q, nullptr, -1.0, rr, main));
         TRYB(blas_axpby(op, p, pv, r, nullptr, 1.0, nullptr, nullptr, 0.0, nullptr, main));
         batch_check_kernel<<<1, 64, 0, main>>>(nv, rr, nb, tol2, act, dstate + i, 0, 0, 0);
@@ -194,33 +185,31 @@ extern "C" int dirac_solve_batched(int nsolves, dirac_op *const *ops, const void
     {
         // one segment (K iterations + recompute + convergence check) of solve i on stream s
         auto record_segment = [&](int i, cudaStream_t s, cudaGraphConditionalHandle cond, int set_cond) -> int {
-            const dirac_op *op = ops[i];
+            const dirac_op *op = &views[i];
             const dirac_prec p = op->prec;
             const int nv = op->nv;
             void *r = vecs[i * 4 + 0], *pv = vecs[i * 4 + 1], *q = vecs[i * 4 + 2], *rhs = vecs[i * 4 + 3];
-            double *sc = scal[i];
-            double *rr = sc, *rr_new = sc + 128, *pq = sc + 2 * 128, *alpha = sc + 3 * 128, *beta = sc + 4 * 128;
-            double *act = sc + 5 * 128, *nb = sc + 6 * 128;
+            const CgScalars &c = scal[i];
+            double *rr_new = c.best;   // free: no stop rule uses it
             int e;
             for (int k = 0; k < K; ++k) {
-                if ((e = batch_apply_A_pq(op, pv, q, pq, m0[i], s))) return e;
-                batch_alpha_kernel<<<1, 64, 0, s>>>(nv, rr, pq, act, alpha);
-                if ((e = blas_axpby(op, p, r, r, nullptr, 1.0, q, alpha, -1.0, rr_new, s))) return e;
+                if ((e = solver_cg_step(op, pv, q, m0[i], c, s))) return e;
+                if ((e = blas_cg_residual(op, p, r, q, c, s))) return e;
                 if (k + 1 < K) {
-                    batch_beta_kernel<<<1, 64, 0, s>>>(nv, rr_new, rr, act, beta);
-                    if ((e = blas_update_xp(op, p, x[i], pv, r, alpha, beta, s))) return e;   // x += alpha p; p = r + beta p
+                    if ((e = blas_cg_update(op, p, xi[i], pv, r, c, s))) return e;   // x += alpha p; p = r + beta p
                 } else {
                     // last iteration of the segment: x += alpha p, then replace r by
                     // the true residual and build the next direction from it
-                    if ((e = blas_axpby(op, p, x[i], x[i], nullptr, 1.0, pv, alpha, 1.0, nullptr, s))) return e;
-                    if ((e = op_apply_cg(op, x[i], q, m0[i], s))) return e;
+                    if ((e = blas_axpby(op, p, xi[i], xi[i], nullptr, 1.0, pv, c.alpha, 1.0, nullptr, s))) return e;
+                    if ((e = op_apply_cg(op, xi[i], q, m0[i], s))) return e;
                     if ((e = blas_axpby(op, p, r, rhs, nullptr, 1.0, q, nullptr, -1.0, rr_new, s))) return e;
-                    batch_beta_kernel<<<1, 64, 0, s>>>(nv, rr_new, rr, act, beta);
-                    if ((e = blas_axpby(op, p, pv, r, nullptr, 1.0, pv, beta, 1.0, nullptr, s))) return e;
+                    if ((e = solver_cg_beta(op, rr_new, c, s))) return e;
+                    if ((e = blas_axpby(op, p, pv, r, nullptr, 1.0, pv, c.beta, 1.0, nullptr, s))) return e;
                 }
             }
             // freeze converged RHS (rr now holds the true residual), stamp completion
-            batch_check_kernel<<<1, 64, 0, s>>>(nv, rr, nb, tol2, act, dstate + i, K, cond, set_cond);
+            batch_check_kernel<<<1, 64, 0, s>>>(nv, c.rr, c.nb, tol2, const_cast<double *>(c.act), dstate + i, K, cond,
+                                                set_cond);
             return launch_check("batch segment");
         };
 
@@ -341,6 +330,11 @@ extern "C" int dirac_solve_batched(int nsolves, dirac_op *const *ops, const void
             graph = nullptr;
         }
     }
+    for (int i = 0; i < nsolves; ++i)
+        if (xi[i] != x[i])
+            TRYB(blas_convert_layout(ops[i], xi[i], ops[i]->prec, DIRAC_LAYOUT_SITE_INNER, x[i], ops[i]->prec,
+                                     ops[i]->geom.layout, main));
+    TRYB(cuda_check(cudaStreamSynchronize(main), "batch sync"));
     TRYB(cuda_check(cudaMemcpy(&hstart, dstart, sizeof(hstart), cudaMemcpyDeviceToHost), "D2H stamp"));
     if (stats) {
         const double wall = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
@@ -349,8 +343,8 @@ extern "C" int dirac_solve_batched(int nsolves, dirac_op *const *ops, const void
             memset(&st, 0, sizeof(st));
             const int nv = ops[i]->nv;
             double rr[64], nb[64];
-            TRYB(cuda_check(cudaMemcpy(rr, scal[i], nv * sizeof(double), cudaMemcpyDeviceToHost), "D2H"));
-            TRYB(cuda_check(cudaMemcpy(nb, scal[i] + 6 * 128, nv * sizeof(double), cudaMemcpyDeviceToHost), "D2H"));
+            TRYB(cuda_check(cudaMemcpy(rr, scal[i].rr, nv * sizeof(double), cudaMemcpyDeviceToHost), "D2H"));
+            TRYB(cuda_check(cudaMemcpy(nb, scal[i].nb, nv * sizeof(double), cudaMemcpyDeviceToHost), "D2H"));
             st.iters = hstate[i].iters;
             st.recomputes = hstate[i].iters / K;
             st.status = hstate[i].done ? DIRAC_OK : DIRAC_NOT_CONVERGED;

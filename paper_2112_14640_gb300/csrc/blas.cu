@@ -32,76 +32,25 @@ inline int blas_group(dirac_prec p, int nv) { return pick_vr(p, nv); }
 // Threads per block: a multiple of the number of column groups nv/G.
 inline int red_block(int ngroups) { return ngroups * (kRedThreads / ngroups); }
 
-// Reduce the per-thread column sums vals[G][NOUT] over the R row-threads of the
-// block (fixed pairwise tree) and store the block's partial sums for its nv
-// columns: partial_block[v][NOUT].
-template <int G, int NOUT>
-__device__ __forceinline__ void block_reduce_store(const double (&vals)[G][NOUT], double *sh, int r, int vg, int R,
-                                                   int ng, double *partial_block) {
-    constexpr int W = G * NOUT;
-#pragma unroll
-    for (int i = 0; i < G; ++i)
-#pragma unroll
-        for (int q = 0; q < NOUT; ++q) sh[(r * ng + vg) * W + i * NOUT + q] = vals[i][q];
-    __syncthreads();
-    for (int off = 1; off < R; off *= 2) {
-        if ((r % (2 * off)) == 0 && r + off < R) {
-#pragma unroll
-            for (int w = 0; w < W; ++w) sh[(r * ng + vg) * W + w] += sh[((r + off) * ng + vg) * W + w];
-        }
-        __syncthreads();
-    }
-    if (r == 0) {
-#pragma unroll
-        for (int i = 0; i < G; ++i)
-#pragma unroll
-            for (int q = 0; q < NOUT; ++q) partial_block[(vg * G + i) * NOUT + q] = sh[vg * W + i * NOUT + q];
-    }
-}
-
-// Second pass of a reduction: partial[b][col] (col = v*NOUT + q, cols =
-// nv*NOUT) -> out[col].  One block of kFinThreads threads: T = kFinThreads /
-// cols threads per column each sum the blocks t, t+T, ... in order, then a
-// fixed pairwise tree combines the T partial sums, so the result does not
-// depend on timing.  KEEP = 1 keeps only q = 0 of each v (the real part of a
-// dot product) and writes out[v].
-constexpr int kFinThreads = 256;
-template <int NOUT, int KEEP>
-__global__ void __launch_bounds__(kFinThreads) finalize_kernel(const double *__restrict__ partial, int nblocks,
-                                                               int nv, double *__restrict__ out) {
-    __shared__ double sh[kFinThreads];
-    const int cols = nv * KEEP;
-    const int T = kFinThreads / cols;
-    const int t = threadIdx.x / cols, c = threadIdx.x % cols;
-    // column c of the output is column src of the partials
-    const int src = KEEP == NOUT ? c : c * NOUT;
-    double acc = 0.0;
-    if (t < T)
-        for (int b = t; b < nblocks; b += T) acc += partial[(long long)b * nv * NOUT + src];
-    sh[threadIdx.x] = acc;
-    __syncthreads();
-    for (int off = 1; off < T; off *= 2) {
-        if (t % (2 * off) == 0 && t + off < T) sh[t * cols + c] += sh[(t + off) * cols + c];
-        __syncthreads();
-    }
-    if (t == 0) out[c] = sh[c];
-}
-
 // Per-thread accumulator of a real sum.  FP64 data: a plain double.  FP32
 // data: (s, c) with the exact value s + c of everything added so far up to
 // the errors of the error-free steps (Knuth's two-sum and Dekker's product via
 // FMA); the explicit __f*_rn intrinsics keep the compiler from contracting or
-// reassociating them.
+// reassociating them.  Either is eight bytes, and two of them join without
+// leaving the FP32 pipe, so a block's and a launch's partial sums stay in this
+// form: FP64 additions of every thread's sum cost as much as a small reduction.
 template <typename A>
 struct RedAcc;
 template <>
 struct RedAcc<double> {
     double s = 0.0;
     __device__ __forceinline__ void mac(double x, double y) { s = fma(x, y, s); }
+    __device__ __forceinline__ void join(const RedAcc &o) { s += o.s; }
+    __device__ __forceinline__ RedAcc down(int lanes) const { return RedAcc{__shfl_down_sync(~0u, s, lanes)}; }
     __device__ __forceinline__ double value() const { return s; }
 };
 template <>
-struct RedAcc<float> {
+struct __align__(8) RedAcc<float> {
     float s = 0.f, c = 0.f;
     __device__ __forceinline__ void add(float p) {
         const float t = __fadd_rn(s, p);
@@ -114,8 +63,77 @@ struct RedAcc<float> {
         add(p);
         c = __fadd_rn(c, __fmaf_rn(x, y, -p));
     }
+    __device__ __forceinline__ void join(const RedAcc &o) {
+        add(o.s);
+        c = __fadd_rn(c, o.c);
+    }
+    __device__ __forceinline__ RedAcc down(int lanes) const {
+        return RedAcc{__shfl_down_sync(~0u, s, lanes), __shfl_down_sync(~0u, c, lanes)};
+    }
     __device__ __forceinline__ double value() const { return (double)s + (double)c; }
 };
+
+// Rows of a column in shared memory: [column][row], an odd pitch.
+__host__ __device__ constexpr int red_pitch(int rows) { return rows | 1; }
+
+// Join the `rows` sums of every column, one warp per column at a time: lanes
+// take rows lane, lane + 32, ..., then a fixed tree; put(column, sum) runs in
+// lane 0.  Whole warps only (blocks need not be a multiple of 32 threads).
+template <typename A, typename PUT>
+__device__ __forceinline__ void join_columns(const RedAcc<A> *sh, int cols, int rows, PUT put) {
+    const int nwarps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp >= nwarps) return;
+    for (int c = warp; c < cols; c += nwarps) {
+        RedAcc<A> acc;
+        for (int r = lane; r < rows; r += 32) acc.join(sh[c * red_pitch(rows) + r]);
+        for (int off = 16; off > 0; off /= 2) acc.join(acc.down(off));
+        if (lane == 0) put(c, acc);
+    }
+}
+
+// The sums vals[G][NOUT] of the R row-threads of a block, joined per column
+// and stored as the block's row of partial sums: partial_block[v NOUT + q].
+template <int G, int NOUT, typename A>
+__device__ __forceinline__ void block_reduce_store(const RedAcc<A> (&vals)[G][NOUT], RedAcc<A> *sh, int r, int vg, int R,
+                                                   int ng, RedAcc<A> *partial_block) {
+    if (r < R)
+#pragma unroll
+        for (int i = 0; i < G; ++i)
+#pragma unroll
+            for (int q = 0; q < NOUT; ++q) sh[((vg * G + i) * NOUT + q) * red_pitch(R) + r] = vals[i][q];
+    __syncthreads();
+    join_columns(sh, ng * G * NOUT, R, [&](int c, const RedAcc<A> &v) { partial_block[c] = v; });
+}
+
+// Second pass of a reduction: partial[b][col] (col = v*NOUT + q, cols =
+// nv*NOUT) -> out[col].  One block of kFinThreads threads: T = kFinThreads /
+// cols threads per column each join the blocks t, t+T, ... in order, then the
+// T sums, so the result does not depend on timing.
+constexpr int kFinThreads = 256;
+template <int NOUT, typename A>
+__global__ void __launch_bounds__(kFinThreads) finalize_kernel(const RedAcc<A> *__restrict__ partial, int nblocks,
+                                                               int nv, double *__restrict__ out) {
+    __shared__ double raw[2 * kFinThreads];   // cols rows of T | 1
+    RedAcc<A> *sh = reinterpret_cast<RedAcc<A> *>(raw);
+    const int cols = nv * NOUT;
+    const int T = kFinThreads / cols;
+    const int t = threadIdx.x / cols, c = threadIdx.x % cols;
+    RedAcc<A> acc;
+    if (t < T) {
+        constexpr int U = 8;   // rows in flight per thread
+        for (int b0 = t; b0 < nblocks; b0 += U * T) {
+            RedAcc<A> in[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (b0 + u * T < nblocks) in[u] = partial[(long long)(b0 + u * T) * cols + c];
+#pragma unroll
+            for (int u = 0; u < U; ++u) acc.join(in[u]);   // zero past the last row
+        }
+        sh[c * red_pitch(T) + t] = acc;
+    }
+    __syncthreads();
+    join_columns(sh, cols, T, [&](int col, const RedAcc<A> &v) { out[col] = v.value(); });
+}
 
 // thread (r, vg) of a block walks the rows r0 = block*R + r, stride grid*R and
 // owns columns vg*G .. vg*G+G-1
@@ -137,17 +155,19 @@ struct RowMap {
 };
 
 template <typename E, int G>
-__global__ void norm2_kernel(const E *__restrict__ x, long long rows, int nv, double *__restrict__ partial,
+__global__ void norm2_kernel(const E *__restrict__ x, long long rows, int nv,
+                             RedAcc<typename Acc<E>::T> *__restrict__ partial,
                              RowMap rm = RowMap{}) {
-    extern __shared__ double sh[];
+    extern __shared__ __align__(8) unsigned char red_smem[];
     using A = typename Acc<E>::T;
+    RedAcc<A> *sh = reinterpret_cast<RedAcc<A> *>(red_smem);
     BLAS_THREAD_SETUP
-    RedAcc<A> acc[G];
+    RedAcc<A> acc[G][1];
     auto add = [&](const cx<A> (&a)[G]) {
 #pragma unroll
         for (int i = 0; i < G; ++i) {
-            acc[i].mac(a[i].re, a[i].re);
-            acc[i].mac(a[i].im, a[i].im);
+            acc[i][0].mac(a[i].re, a[i].re);
+            acc[i][0].mac(a[i].im, a[i].im);
         }
     };
     if (live) {
@@ -165,26 +185,24 @@ __global__ void norm2_kernel(const E *__restrict__ x, long long rows, int nv, do
             add(a[0]);
         }
     }
-    double out[G][1];
-#pragma unroll
-    for (int i = 0; i < G; ++i) out[i][0] = acc[i].value();
-    block_reduce_store<G, 1>(out, sh, r, vg, R, ng, partial + (long long)blockIdx.x * nv);
+    block_reduce_store<G, 1, A>(acc, sh, r, vg, R, ng, partial + (long long)blockIdx.x * nv);
 }
 
 template <typename E, int G>
 __global__ void dot_kernel(const E *__restrict__ x, const E *__restrict__ y, long long rows, int nv,
-                           double *__restrict__ partial, RowMap rm = RowMap{}) {
-    extern __shared__ double sh[];
+                           RedAcc<typename Acc<E>::T> *__restrict__ partial, RowMap rm = RowMap{}) {
+    extern __shared__ __align__(8) unsigned char red_smem[];
     using A = typename Acc<E>::T;
+    RedAcc<A> *sh = reinterpret_cast<RedAcc<A> *>(red_smem);
     BLAS_THREAD_SETUP
-    RedAcc<A> re[G], im[G];
+    RedAcc<A> acc[G][2];
     auto add = [&](const cx<A> (&a)[G], const cx<A> (&b)[G]) {
 #pragma unroll
         for (int i = 0; i < G; ++i) {   // conj(x) * y
-            re[i].mac(a[i].re, b[i].re);
-            re[i].mac(a[i].im, b[i].im);
-            im[i].mac(a[i].re, b[i].im);
-            im[i].mac(-a[i].im, b[i].re);
+            acc[i][0].mac(a[i].re, b[i].re);
+            acc[i][0].mac(a[i].im, b[i].im);
+            acc[i][1].mac(a[i].re, b[i].im);
+            acc[i][1].mac(-a[i].im, b[i].re);
         }
     };
     if (live) {
@@ -208,13 +226,7 @@ __global__ void dot_kernel(const E *__restrict__ x, const E *__restrict__ y, lon
             add(a[0], b[0]);
         }
     }
-    double out[G][2];
-#pragma unroll
-    for (int i = 0; i < G; ++i) {
-        out[i][0] = re[i].value();
-        out[i][1] = im[i].value();
-    }
-    block_reduce_store<G, 2>(out, sh, r, vg, R, ng, partial + 2LL * blockIdx.x * nv);
+    block_reduce_store<G, 2, A>(acc, sh, r, vg, R, ng, partial + 2LL * blockIdx.x * nv);
 }
 
 template <typename A>
@@ -227,9 +239,11 @@ __device__ __forceinline__ cx<A> coef(const double *c, double scale, int v) {
 // or y.  With partial != null also reduces |z|^2 per column.
 template <typename E, int G>
 __global__ void axpby_kernel(E *z, const E *x, const E *y, const double *__restrict__ ac, double as,
-                             const double *__restrict__ bc, double bs, long long rows, int nv, double *partial) {
-    extern __shared__ double sh[];
+                             const double *__restrict__ bc, double bs, long long rows, int nv,
+                             RedAcc<typename Acc<E>::T> *partial) {
+    extern __shared__ __align__(8) unsigned char red_smem[];
     using A = typename Acc<E>::T;
+    RedAcc<A> *sh = reinterpret_cast<RedAcc<A> *>(red_smem);
     BLAS_THREAD_SETUP
     cx<A> a[G], b[G];
 #pragma unroll
@@ -237,7 +251,7 @@ __global__ void axpby_kernel(E *z, const E *x, const E *y, const double *__restr
         a[i] = coef<A>(ac, as, vg * G + i);
         b[i] = coef<A>(bc, bs, vg * G + i);
     }
-    RedAcc<A> acc[G];
+    RedAcc<A> acc[G][1];
     // one row: combine, store, and (optionally) add |z|^2 of the value as
     // stored: the registers rounded through the storage type (z may alias x
     // or y, so it is not re-read)
@@ -255,8 +269,8 @@ __global__ void axpby_kernel(E *z, const E *x, const E *y, const double *__restr
             for (int i = 0; i < G; ++i) {
                 const A re = (A)to_acc<E>(from_acc<E, A>(out[i].re));
                 const A im = (A)to_acc<E>(from_acc<E, A>(out[i].im));
-                acc[i].mac(re, re);
-                acc[i].mac(im, im);
+                acc[i][0].mac(re, re);
+                acc[i][0].mac(im, im);
             }
         }
     };
@@ -282,58 +296,229 @@ __global__ void axpby_kernel(E *z, const E *x, const E *y, const double *__restr
         }
     }
     if (partial) {
-        double out[G][1];
-#pragma unroll
-        for (int i = 0; i < G; ++i) out[i][0] = acc[i].value();
-        block_reduce_store<G, 1>(out, sh, r, vg, R, ng, partial + (long long)blockIdx.x * nv);
+        block_reduce_store<G, 1, A>(acc, sh, r, vg, R, ng, partial + (long long)blockIdx.x * nv);
     }
 }
 
-// The two Krylov updates that use the old search direction, in one pass:
-// x += a p, then p = r + b p.
+// ------------------------------------------------------------ CG kernels
+// The three vector passes of a CG iteration with the scalar work between them
+// done by the last block of the pass that produces its input: one launch each
+// where a pass, its reduction's second stage and a coefficient kernel were
+// three, and no value the host has to see before the next launch.  The
+// iterations that the host enqueues ahead of the stop rule do nothing once it
+// has been met (ctl[0]).  Memory-bound on large lattices (16^3x32, D_W,
+// N_v = 4, FP32: dot 16, residual 26, update 42 us; the update moves 250 MB at
+// 6 TB/s), bound by the chain load - reduce - last block on small ones (8^4,
+// N_v = 3: about 5, 6 and 3 us).
+
+// Join the blocks' partial rows (nv sums each) in the last block to arrive;
+// the N_v values there, null in every other block.  Fixed order, so
+// reproducible.  This block's row was written before the call.
+__device__ __forceinline__ RedAcc<double> load_cg(const RedAcc<double> *p) {
+    return RedAcc<double>{__ldcg(reinterpret_cast<const double *>(p))};
+}
+__device__ __forceinline__ RedAcc<float> load_cg(const RedAcc<float> *p) {
+    const float2 f = __ldcg(reinterpret_cast<const float2 *>(p));
+    return RedAcc<float>{f.x, f.y};
+}
+template <typename A>
+__device__ __forceinline__ const double *last_block_sum(const RedAcc<A> *partial, unsigned *counter, int nv,
+                                                        RedAcc<A> *sh) {
+    __shared__ bool last;
+    __shared__ double sums[64];
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicInc(counter, gridDim.x - 1) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return nullptr;
+    __threadfence();
+    const int T = blockDim.x / nv, t = threadIdx.x / nv, c = threadIdx.x - t * nv;
+    if (t < T) {
+        RedAcc<A> acc;
+        constexpr int U = 8;   // rows in flight per thread
+        for (int b0 = t; b0 < (int)gridDim.x; b0 += U * T) {
+            RedAcc<A> in[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (b0 + u * T < (int)gridDim.x) in[u] = load_cg(partial + (long long)(b0 + u * T) * nv + c);
+#pragma unroll
+            for (int u = 0; u < U; ++u) acc.join(in[u]);   // zero past the last row
+        }
+        sh[c * red_pitch(T) + t] = acc;
+    }
+    __syncthreads();
+    join_columns(sh, nv, T, [&](int col, const RedAcc<A> &v) { sums[col] = v.value(); });
+    __syncthreads();
+    return sums;
+}
+
+__device__ __forceinline__ bool cg_stopped(const CgScalars &k) { return k.ctl && *(volatile int *)k.ctl; }
+
 template <typename E, int G>
-__global__ void update_xp_kernel(E *x, E *p, const E *__restrict__ r_, const double *__restrict__ ac,
-                                 const double *__restrict__ bc, long long rows, int nv) {
+__global__ void cg_dot_kernel(const E *__restrict__ x, const E *__restrict__ y, long long rows, int nv, CgScalars k) {
+    extern __shared__ __align__(8) unsigned char red_smem[];
     using A = typename Acc<E>::T;
+    RedAcc<A> *sh = reinterpret_cast<RedAcc<A> *>(red_smem);
+    if (cg_stopped(k)) return;
+    BLAS_THREAD_SETUP
+    RedAcc<A> acc[G][1];
+    auto add = [&](const cx<A> (&a)[G], const cx<A> (&b)[G]) {
+#pragma unroll
+        for (int i = 0; i < G; ++i) {
+            acc[i][0].mac(a[i].re, b[i].re);
+            acc[i][0].mac(a[i].im, b[i].im);
+        }
+    };
+    if (live)
+        for (long long row = (long long)blockIdx.x * R + r; row < rows; row += 4 * stride) {
+            cx<A> a[4][G], b[4][G];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const long long e = 2 * ((row + u * stride) * nv + vg * G);
+                if (row + u * stride < rows) {
+                    load_cx<E, G, A>(x + e, a[u]);
+                    load_cx<E, G, A>(y + e, b[u]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (row + u * stride < rows) add(a[u], b[u]);
+        }
+    RedAcc<A> *partial = reinterpret_cast<RedAcc<A> *>(k.partial);
+    block_reduce_store<G, 1, A>(acc, sh, r, vg, R, ng, partial + (long long)blockIdx.x * nv);
+    const double *sums = last_block_sum(partial, k.counter, nv, sh);
+    if (!sums) return;
+    const int v = threadIdx.x;
+    if (v >= nv) return;
+    const double pq = sums[v];
+    const bool go = k.act[v] != 0.0 && (k.positive ? pq > 0.0 : pq != 0.0);
+    k.pq[v] = pq;
+    k.alpha[2 * v] = go ? k.rr[v] / pq : 0.0;
+    k.alpha[2 * v + 1] = 0.0;
+}
+
+template <typename E, int G>
+__global__ void cg_residual_kernel(E *rv, const E *__restrict__ q, long long rows, int nv, CgScalars k) {
+    extern __shared__ __align__(8) unsigned char red_smem[];
+    using A = typename Acc<E>::T;
+    RedAcc<A> *sh = reinterpret_cast<RedAcc<A> *>(red_smem);
+    if (cg_stopped(k)) return;
+    BLAS_THREAD_SETUP
+    A a[G];
+#pragma unroll
+    for (int i = 0; i < G; ++i) a[i] = live ? (A)(-k.alpha[2 * (vg * G + i)]) : (A)0;
+    RedAcc<A> acc[G][1];
+    // |r|^2 of the value as stored (rounded through the storage type)
+    auto finish = [&](long long e, const cx<A> (&tr)[G], const cx<A> (&tq)[G]) {
+        cx<A> o[G];
+#pragma unroll
+        for (int i = 0; i < G; ++i) {
+            o[i] = cx<A>{fma(a[i], tq[i].re, tr[i].re), fma(a[i], tq[i].im, tr[i].im)};
+            const A re = (A)to_acc<E>(from_acc<E, A>(o[i].re));
+            const A im = (A)to_acc<E>(from_acc<E, A>(o[i].im));
+            acc[i][0].mac(re, re);
+            acc[i][0].mac(im, im);
+        }
+        store_cx<E, G, A>(rv + e, o);
+    };
+    if (live)
+        for (long long row = (long long)blockIdx.x * R + r; row < rows; row += 4 * stride) {
+            cx<A> tr[4][G], tq[4][G];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const long long e = 2 * ((row + u * stride) * nv + vg * G);
+                if (row + u * stride < rows) {
+                    load_cx<E, G, A>(rv + e, tr[u]);
+                    load_cx<E, G, A>(q + e, tq[u]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (row + u * stride < rows) finish(2 * ((row + u * stride) * nv + vg * G), tr[u], tq[u]);
+        }
+    RedAcc<A> *partial = reinterpret_cast<RedAcc<A> *>(k.partial);
+    block_reduce_store<G, 1, A>(acc, sh, r, vg, R, ng, partial + (long long)blockIdx.x * nv);
+    const double *sums = last_block_sum(partial, k.counter, nv, sh);
+    if (!sums) return;
+    const int v = threadIdx.x;
+    bool bad = false, pass = true, trip = false;
+    if (v < nv) {
+        const double rn = sums[v], ro = k.rr[v];
+        const bool on = k.act[v] != 0.0;
+        k.rr_prev[v] = ro;
+        k.rr[v] = rn;
+        k.beta[2 * v] = on && (k.positive ? ro > 0.0 : ro != 0.0) ? rn / ro : 0.0;
+        k.beta[2 * v + 1] = 0.0;
+        if (k.rule != CgScalars::kNone) {
+            double *h = k.hist + (long long)k.ctl[1] * 3 * nv;
+            h[v] = k.pq[v];
+            h[nv + v] = ro;
+            h[2 * nv + v] = rn;
+            bad = !isfinite(rn);
+            const double rnorm = sqrt(rn), goal = k.tol * sqrt(k.nb[v]);
+            if (k.rule == CgScalars::kPlain) {
+                pass = !on || rnorm < goal;
+            } else {
+                if (on) {
+                    if (rnorm < k.best[v]) {
+                        k.best[v] = rnorm;
+                        k.since[v] = 0.0;
+                    } else {
+                        k.since[v] += 1.0;
+                        trip = k.since[v] >= k.stall;
+                    }
+                    trip = trip || rnorm < k.delta * k.rmax[v] || rnorm < goal * k.sig[v];
+                }
+                k.rmax[v] = fmax(k.rmax[v], rnorm);
+            }
+        }
+    }
+    if (k.rule == CgScalars::kNone) return;
+    const bool any_bad = __syncthreads_or(bad), any_trip = __syncthreads_or(trip);
+    const bool all_pass = __syncthreads_and(pass);
+    if (threadIdx.x == 0) {
+        k.ctl[1] += 1;
+        k.ctl[2] = 1;
+        k.ctl[0] = any_bad || (k.rule == CgScalars::kPlain ? all_pass : any_trip);
+    }
+}
+
+// x += alpha p, then p = r + beta p (real coefficients)
+template <typename E, int G>
+__global__ void cg_update_kernel(E *x, E *p, const E *__restrict__ r_, long long rows, int nv, CgScalars k) {
+    using A = typename Acc<E>::T;
+    if (cg_stopped(k) || (k.ctl && k.ctl[2] == 0)) return;
     BLAS_THREAD_SETUP
     if (!live) return;
-    cx<A> a[G], b[G];
+    A a[G], b[G];
 #pragma unroll
     for (int i = 0; i < G; ++i) {
-        a[i] = coef<A>(ac, 1.0, vg * G + i);
-        b[i] = coef<A>(bc, 1.0, vg * G + i);
+        a[i] = (A)k.alpha[2 * (vg * G + i)];
+        b[i] = (A)k.beta[2 * (vg * G + i)];
     }
     auto finish = [&](long long e, cx<A> (&xv)[G], cx<A> (&pv)[G], const cx<A> (&rv)[G]) {
 #pragma unroll
         for (int i = 0; i < G; ++i) {
-            cmac(xv[i], a[i], pv[i]);
-            cx<A> np = rv[i];
-            cmac(np, b[i], pv[i]);
-            pv[i] = np;
+            rmac(xv[i], a[i], pv[i]);
+            pv[i] = cx<A>{fma(b[i], pv[i].re, rv[i].re), fma(b[i], pv[i].im, rv[i].im)};
         }
         store_cx<E, G, A>(x + e, xv);
         store_cx<E, G, A>(p + e, pv);
     };
-    long long row = (long long)blockIdx.x * R + r;
-    for (; row + 3 * stride < rows; row += 4 * stride) {
+    for (long long row = (long long)blockIdx.x * R + r; row < rows; row += 4 * stride) {
         cx<A> xv[4][G], pv[4][G], rv[4][G];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const long long e = 2 * ((row + u * stride) * nv + vg * G);
-            load_cx<E, G, A>(x + e, xv[u]);
-            load_cx<E, G, A>(p + e, pv[u]);
-            load_cx<E, G, A>(r_ + e, rv[u]);
+            if (row + u * stride < rows) {
+                load_cx<E, G, A>(x + e, xv[u]);
+                load_cx<E, G, A>(p + e, pv[u]);
+                load_cx<E, G, A>(r_ + e, rv[u]);
+            }
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) finish(2 * ((row + u * stride) * nv + vg * G), xv[u], pv[u], rv[u]);
-    }
-    for (; row < rows; row += stride) {
-        const long long e = 2 * (row * nv + vg * G);
-        cx<A> xv[1][G], pv[1][G], rv[1][G];
-        load_cx<E, G, A>(x + e, xv[0]);
-        load_cx<E, G, A>(p + e, pv[0]);
-        load_cx<E, G, A>(r_ + e, rv[0]);
-        finish(e, xv[0], pv[0], rv[0]);
+        for (int u = 0; u < 4; ++u)
+            if (row + u * stride < rows) finish(2 * ((row + u * stride) * nv + vg * G), xv[u], pv[u], rv[u]);
     }
 }
 
@@ -391,6 +576,39 @@ __global__ void convert_kernel(const S *__restrict__ src, D *__restrict__ dst, l
     if (i < count) dst[i] = from_acc<D, typename Acc<S>::T>(to_acc<S>(src[i]));
 }
 
+// A vector in the other layout (and precision): one thread per complex number
+// in the order of dst.  inner: dst is [cs][site][v], src [site][cs][v]; else
+// the reverse.
+template <typename S, typename D>
+__global__ void __launch_bounds__(256) relayout_kernel(const S *__restrict__ src, D *__restrict__ dst, long long V,
+                                                       int ncs, int nv, int inner) {
+    using A = typename Acc<S>::T;
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= V * ncs * nv) return;
+    long long row;   // the pair (site, cs) in dst's order
+    int v;
+    split_tid(i, nv, row, v);
+    long long o;
+    if (inner) {
+        const long long cs = row / V;
+        o = (row - cs * V) * ncs + cs;
+    } else {
+        long long site;
+        int cs;
+        split_tid(row, ncs, site, cs);
+        o = cs * V + site;
+    }
+    const cx<A> z = ld1<S, A>(src + 2 * (o * nv + v));
+    const D e[2] = {from_acc<D, A>(z.re), from_acc<D, A>(z.im)};
+    if constexpr (sizeof(D) == 8) {
+        *reinterpret_cast<double2 *>(dst + 2 * i) = double2{e[0], e[1]};
+    } else {
+        typename Raw<2 * (int)sizeof(D)>::T raw;
+        __builtin_memcpy(&raw, e, sizeof(raw));
+        *reinterpret_cast<decltype(raw) *>(dst + 2 * i) = raw;
+    }
+}
+
 // Deterministic pseudo-random fill in [-1, 1) (a 32-bit integer hash of the
 // element index), used to give timing runs realistic, non-zero operands.
 template <typename E>
@@ -418,14 +636,21 @@ int blas_fill_hash(const dirac_op *op, dirac_prec p, void *v, unsigned seed, cud
 
 static inline int red_grid(const dirac_op *op) { return op->red_blocks; }
 
+// the reduction buffer as partial sums of E's accumulators (eight bytes each)
 template <typename E>
-static int launch_norm2(const E *v, long long rows, int nv, dirac_prec p, double *partial, int blocks, double *out,
+static RedAcc<typename Acc<E>::T> *partials(double *buf) {
+    return reinterpret_cast<RedAcc<typename Acc<E>::T> *>(buf);
+}
+
+template <typename E>
+static int launch_norm2(const E *v, long long rows, int nv, dirac_prec p, double *buf, int blocks, double *out,
                         cudaStream_t s) {
+    auto *partial = partials<E>(buf);
     const RedLaunch L = red_launch(p, nv, 1);
     return dispatch_group(L.G, [&](auto gc) {
         constexpr int G = decltype(gc)::value;
         norm2_kernel<E, G><<<blocks, L.tb, L.sh, s>>>(v, rows, nv, partial);
-        finalize_kernel<1, 1><<<1, kFinThreads, 0, s>>>(partial, blocks, nv, out);
+        finalize_kernel<1><<<1, kFinThreads, 0, s>>>(partial, blocks, nv, out);
         return launch_check("norm2_kernel");
     });
 }
@@ -444,22 +669,8 @@ int blas_dot(const dirac_op *op, dirac_prec p, const void *u, const void *v, dou
         return dispatch_group(L.G, [&](auto gc) {
             constexpr int G = decltype(gc)::value;
             dot_kernel<E, G><<<red_grid(op), L.tb, L.sh, s>>>((const E *)u, (const E *)v, op->rows, op->nv,
-                                                              op->red_partial);
-            finalize_kernel<2, 2><<<1, kFinThreads, 0, s>>>(op->red_partial, red_grid(op), op->nv, out);
-            return launch_check("dot_kernel");
-        });
-    });
-}
-
-int blas_dot_re(const dirac_op *op, dirac_prec p, const void *u, const void *v, double *out, cudaStream_t s) {
-    return dispatch_prec(p, [&](auto tag) {
-        using E = std::remove_pointer_t<decltype(tag)>;
-        const RedLaunch L = red_launch(p, op->nv, 2);
-        return dispatch_group(L.G, [&](auto gc) {
-            constexpr int G = decltype(gc)::value;
-            dot_kernel<E, G><<<red_grid(op), L.tb, L.sh, s>>>((const E *)u, (const E *)v, op->rows, op->nv,
-                                                              op->red_partial);
-            finalize_kernel<2, 1><<<1, kFinThreads, 0, s>>>(op->red_partial, red_grid(op), op->nv, out);
+                                                              partials<E>(op->red_partial));
+            finalize_kernel<2><<<1, kFinThreads, 0, s>>>(partials<E>(op->red_partial), red_grid(op), op->nv, out);
             return launch_check("dot_kernel");
         });
     });
@@ -491,8 +702,8 @@ int blas_norm2_range(const dirac_op *op, dirac_prec p, const void *v, long long 
         return dispatch_group(L.G, [&](auto gc) {
             constexpr int G = decltype(gc)::value;
             norm2_kernel<E, G><<<red_grid(op), L.tb, L.sh, s>>>((const E *)v + 2 * first * op->nv, rows, op->nv,
-                                                                op->red_partial, rm);
-            finalize_kernel<1, 1><<<1, kFinThreads, 0, s>>>(op->red_partial, red_grid(op), op->nv, out);
+                                                                partials<E>(op->red_partial), rm);
+            finalize_kernel<1><<<1, kFinThreads, 0, s>>>(partials<E>(op->red_partial), red_grid(op), op->nv, out);
             return launch_check("norm2_kernel");
         });
     });
@@ -510,8 +721,8 @@ int blas_dot_range(const dirac_op *op, dirac_prec p, const void *u, const void *
             constexpr int G = decltype(gc)::value;
             dot_kernel<E, G><<<red_grid(op), L.tb, L.sh, s>>>((const E *)u + 2 * first * op->nv,
                                                               (const E *)v + 2 * first * op->nv, rows, op->nv,
-                                                              op->red_partial, rm);
-            finalize_kernel<2, 2><<<1, kFinThreads, 0, s>>>(op->red_partial, red_grid(op), op->nv, out);
+                                                              partials<E>(op->red_partial), rm);
+            finalize_kernel<2><<<1, kFinThreads, 0, s>>>(partials<E>(op->red_partial), red_grid(op), op->nv, out);
             return launch_check("dot_kernel");
         });
     });
@@ -526,8 +737,8 @@ int blas_axpby(const dirac_op *op, dirac_prec p, void *z, const void *x, const d
             constexpr int G = decltype(gc)::value;
             axpby_kernel<E, G><<<red_grid(op), L.tb, L.sh, s>>>((E *)z, (const E *)x, (const E *)y, a, as, b, bs,
                                                                 op->rows, op->nv,
-                                                                norm_out ? op->red_partial : nullptr);
-            if (norm_out) finalize_kernel<1, 1><<<1, kFinThreads, 0, s>>>(op->red_partial, red_grid(op), op->nv, norm_out);
+                                                                norm_out ? partials<E>(op->red_partial) : nullptr);
+            if (norm_out) finalize_kernel<1><<<1, kFinThreads, 0, s>>>(partials<E>(op->red_partial), red_grid(op), op->nv, norm_out);
             return launch_check("axpby_kernel");
         });
     });
@@ -537,17 +748,50 @@ int blas_axpy(const dirac_op *op, dirac_prec p, const double *alpha, const void 
     return blas_axpby(op, p, y, x, alpha, 1.0, y, nullptr, 1.0, nullptr, s);
 }
 
-int blas_update_xp(const dirac_op *op, dirac_prec p, void *x, void *pv, const void *r, const double *a,
-                   const double *b, cudaStream_t s) {
-    return dispatch_prec(p, [&](auto tag) {
+// Blocks of the CG passes: one row per thread on small lattices, at most
+// kCgBlocks (four per SM: enough loads in flight for the memory rate, and the
+// last block has few partial rows to read).
+static inline int cg_grid(const dirac_op *op, const RedLaunch &L) {
+    const long long want = (op->rows + L.tb / (op->nv / L.G) - 1) / (L.tb / (op->nv / L.G));
+    return (int)(want < kCgBlocks ? want : kCgBlocks);
+}
+
+template <typename F>
+static int dispatch_cg(const dirac_op *op, dirac_prec prec, F &&f) {
+    return dispatch_prec(prec, [&](auto tag) {
         using E = std::remove_pointer_t<decltype(tag)>;
-        const RedLaunch L = red_launch(p, op->nv, 1);
-        return dispatch_group(L.G, [&](auto gc) {
-            constexpr int G = decltype(gc)::value;
-            update_xp_kernel<E, G><<<red_grid(op), L.tb, 0, s>>>((E *)x, (E *)pv, (const E *)r, a, b, op->rows,
-                                                                 op->nv);
-            return launch_check("update_xp_kernel");
-        });
+        const RedLaunch L = red_launch(prec, op->nv, 1);
+        return dispatch_group(L.G, [&](auto gc) { return f((E *)nullptr, gc, L); });
+    });
+}
+
+int blas_cg_dot(const dirac_op *op, dirac_prec prec, const void *p, const void *q, const CgScalars &c,
+                cudaStream_t s) {
+    return dispatch_cg(op, prec, [&](auto tag, auto gc, const RedLaunch &L) {
+        using E = std::remove_pointer_t<decltype(tag)>;
+        cg_dot_kernel<E, decltype(gc)::value><<<cg_grid(op, L), L.tb, L.sh, s>>>((const E *)p, (const E *)q, op->rows,
+                                                                             op->nv, c);
+        return launch_check("cg_dot_kernel");
+    });
+}
+
+int blas_cg_residual(const dirac_op *op, dirac_prec prec, void *r, const void *q, const CgScalars &c,
+                     cudaStream_t s) {
+    return dispatch_cg(op, prec, [&](auto tag, auto gc, const RedLaunch &L) {
+        using E = std::remove_pointer_t<decltype(tag)>;
+        cg_residual_kernel<E, decltype(gc)::value><<<cg_grid(op, L), L.tb, L.sh, s>>>((E *)r, (const E *)q, op->rows,
+                                                                                  op->nv, c);
+        return launch_check("cg_residual_kernel");
+    });
+}
+
+int blas_cg_update(const dirac_op *op, dirac_prec prec, void *x, void *p, const void *r, const CgScalars &c,
+                   cudaStream_t s) {
+    return dispatch_cg(op, prec, [&](auto tag, auto gc, const RedLaunch &L) {
+        using E = std::remove_pointer_t<decltype(tag)>;
+        cg_update_kernel<E, decltype(gc)::value><<<2 * cg_grid(op, L), L.tb, 0, s>>>((E *)x, (E *)p, (const E *)r, op->rows,
+                                                                              op->nv, c);
+        return launch_check("cg_update_kernel");
     });
 }
 
@@ -569,6 +813,21 @@ int blas_convert(const dirac_op *op, const void *src, dirac_prec sp, void *dst, 
             const long long n = op->rows * op->nv * 2;
             convert_kernel<S, D><<<grid_for(n, 256), 256, 0, s>>>((const S *)src, (D *)dst, n);
             return launch_check("convert_kernel");
+        });
+    });
+}
+
+int blas_convert_layout(const dirac_op *op, const void *src, dirac_prec sp, int src_layout, void *dst, dirac_prec dp,
+                        int dst_layout, cudaStream_t s) {
+    if (src_layout == dst_layout) return blas_convert(op, src, sp, dst, dp, s);
+    return dispatch_prec(sp, [&](auto stag) {
+        using S = std::remove_pointer_t<decltype(stag)>;
+        return dispatch_prec(dp, [&](auto dtag) {
+            using D = std::remove_pointer_t<decltype(dtag)>;
+            relayout_kernel<S, D><<<grid_for(op->rows * op->nv, 256), 256, 0, s>>>(
+                (const S *)src, (D *)dst, op->V, (int)(op->rows / op->V), op->nv,
+                dst_layout == DIRAC_LAYOUT_SITE_INNER);
+            return launch_check("relayout_kernel");
         });
     });
 }

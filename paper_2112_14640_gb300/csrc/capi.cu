@@ -108,6 +108,7 @@ static void op_free(dirac_op *op) {
     cudaFree(op->stage_out);
     cudaFree(op->red_partial);
     cudaFree(op->solver_ws);
+    cudaFreeHost(op->solver_host);
     cudaFree(op->force_ws);
     free(op);
 }
@@ -204,7 +205,20 @@ int op_alloc(dirac_kind kind, const dirac_geom *g, dirac_op **out) {
     return DIRAC_OK;
 }
 
-// Lower-precision twin of op (same links/W converted), created once.
+// Links, W and clover blocks are stored alike for both vector layouts, so the
+// view needs no copies; it launches with what was tuned for its own layout.
+dirac_op op_site_inner(const dirac_op *op) {
+    dirac_op view = *op;
+    if (op->geom.layout != DIRAC_LAYOUT_SITE_INNER) {
+        view.geom.layout = DIRAC_LAYOUT_SITE_INNER;
+        view.vr = view.minb = view.block = 0;
+        recall_tuning(&view);
+    }
+    return view;
+}
+
+// Lower-precision twin of op (same links/W converted) on site-inner vectors,
+// created once.
 int op_inner(const dirac_op *op, dirac_prec p, int link_storage, dirac_op **out, cudaStream_t s) {
     if (p == op->prec) {
         *out = (dirac_op *)op;
@@ -216,6 +230,7 @@ int op_inner(const dirac_op *op, dirac_prec p, int link_storage, dirac_op **out,
         dirac_geom g = op->geom;
         g.prec = p;
         g.link_storage = link_storage;
+        g.layout = DIRAC_LAYOUT_SITE_INNER;
         dirac_op *tw = nullptr;
         int rc = op_alloc(op->kind, &g, &tw);
         if (rc) return rc;

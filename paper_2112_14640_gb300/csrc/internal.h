@@ -34,6 +34,7 @@ struct dirac_op {
     int red_blocks;
     void *solver_ws;       // solver workspace (lazy), solver_ws_bytes long
     size_t solver_ws_bytes;
+    double *solver_host;   // pinned copy of a run of CG iterations' scalars (lazy)
     void *force_ws;        // Brillouin force: 216 link terms per site (lazy), force_ws_bytes long
     size_t force_ws_bytes;
     dirac_op *inner[4][2]; // lower-precision twins for mixed solves (lazy), by [prec][link storage]
@@ -257,8 +258,6 @@ int launch_bril_force(dirac_op *op, const void *psi, const void *chi, void *out,
 // BLAS-1 (vectors in precision p with op's shape)
 int blas_norm2(const dirac_op *op, dirac_prec p, const void *v, double *out, cudaStream_t s);
 int blas_dot(const dirac_op *op, dirac_prec p, const void *u, const void *v, double *out, cudaStream_t s);
-// Re <u, v> per column: out[v] (N_v doubles)
-int blas_dot_re(const dirac_op *op, dirac_prec p, const void *u, const void *v, double *out, cudaStream_t s);
 int blas_norm2_range(const dirac_op *op, dirac_prec p, const void *v, long long site0, long long nsites, double *out,
                      cudaStream_t s);
 int blas_dot_range(const dirac_op *op, dirac_prec p, const void *u, const void *v, long long site0, long long nsites,
@@ -268,12 +267,51 @@ int blas_axpy(const dirac_op *op, dirac_prec p, const double *alpha, const void 
 // x or y may be null; z may alias x or y; norm_out (device, nv doubles) receives |z|^2 if non-null.
 int blas_axpby(const dirac_op *op, dirac_prec p, void *z, const void *x, const double *a_coef, double as,
                const void *y, const double *b_coef, double bs, double *norm_out, cudaStream_t s);
-// x += a p, then p = r + b p (a, b per-RHS complex pairs)
-int blas_update_xp(const dirac_op *op, dirac_prec p, void *x, void *pv, const void *r, const double *a,
-                   const double *b, cudaStream_t s);
+// Device scalars of a CG recurrence, nv doubles each unless noted, and the
+// rule by which the device ends a run of iterations that the host enqueued
+// ahead (blas.cu).
+struct CgScalars {
+    double *rr, *rr_prev, *pq, *alpha, *beta;   // alpha, beta: (re, im) pairs, im = 0
+    const double *act;                          // 0: frozen RHS
+    enum Rule { kNone, kPlain, kReliable } rule;
+    bool positive;                              // steps only where <p, A p> and |r|^2 are > 0 (not just nonzero)
+    // kPlain: stop once every active |r| < tol |b|; kReliable: once one falls
+    // below delta rmax or tol |b| sig, or has not improved for `stall`
+    // iterations; both: on a NaN or infinity
+    double tol, delta;
+    int stall;
+    const double *nb, *sig;
+    double *best, *rmax, *since;
+    // [0] stopped, [1] iterations done since both were cleared, [2] an update
+    // of x and p is due (alpha and beta of the last iteration not yet used)
+    int *ctl;
+    double *hist;         // per iteration: <p, A p>, old |r|^2, new |r|^2 (3 nv)
+    double *partial;      // one row of nv doubles per block
+    unsigned *counter;    // zero between launches
+};
+// pq = Re <p, q> and alpha = rr / pq
+int blas_cg_dot(const dirac_op *op, dirac_prec prec, const void *p, const void *q, const CgScalars &c, cudaStream_t s);
+// iterations of history `hist` holds, and the blocks `partial` has rows for
+constexpr int kCgHistory = 20, kCgBlocks = 608;
+// r -= alpha q; rr_prev = rr, rr = |r|^2, beta = rr / rr_prev, history and stop rule
+int blas_cg_residual(const dirac_op *op, dirac_prec prec, void *r, const void *q, const CgScalars &c, cudaStream_t s);
+// x += alpha p, p = r + beta p, if due and not stopped (always where c.ctl is null)
+int blas_cg_update(const dirac_op *op, dirac_prec prec, void *x, void *p, const void *r, const CgScalars &c,
+                   cudaStream_t s);
 int blas_gamma5(const dirac_op *op, dirac_prec p, void *v, cudaStream_t s);
 int blas_fill_hash(const dirac_op *op, dirac_prec p, void *v, unsigned seed, cudaStream_t s);
 int blas_convert(const dirac_op *op, const void *src, dirac_prec sp, void *dst, dirac_prec dp, cudaStream_t s);
+
+// the same between layouts (DIRAC_LAYOUT_*)
+int blas_convert_layout(const dirac_op *op, const void *src, dirac_prec sp, int src_layout, void *dst, dirac_prec dp,
+                        int dst_layout, cudaStream_t s);
+
+// CG scalars of the operator's solver workspace (solver.cu), no stop rule set
+int solver_cg(const dirac_op *op, void **vecs, int nvecs, CgScalars *c, cudaStream_t s);
+// q = A p and alpha = rr / <p, q>
+int solver_cg_step(const dirac_op *op, const void *p, void *q, double m0, const CgScalars &c, cudaStream_t s);
+// beta = rr_new / rr_prev and rr = rr_new, after rr_new was recomputed
+int solver_cg_beta(const dirac_op *op, const double *rr_new, const CgScalars &c, cudaStream_t s);
 
 // operator handle helpers (capi.cu)
 int op_apply(const dirac_op *op, const void *in, void *out, double m0, int sgn, cudaStream_t s);
@@ -282,6 +320,9 @@ int op_apply_normal(const dirac_op *op, const void *in, void *out, double m0, cu
 int op_apply_cg(const dirac_op *op, const void *in, void *out, double m0, cudaStream_t s);
 int op_alloc(dirac_kind kind, const dirac_geom *g, dirac_op **out);
 int op_inner(const dirac_op *op, dirac_prec p, int link_storage, dirac_op **out, cudaStream_t s);
+// The same operator on site-inner vectors, the order the solvers iterate in: a
+// view that shares op's links and buffers and must not outlive the call.
+dirac_op op_site_inner(const dirac_op *op);
 void op_destroy(dirac_op *op);
 
 }  // namespace dgb

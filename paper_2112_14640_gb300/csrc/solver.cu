@@ -14,8 +14,13 @@
 // or at maxit.  An RHS whose recomputed residual passes is frozen
 // (alpha = beta = 0) while the others continue.
 //
-// Per-RHS coefficients are formed on the device from FP64 reductions; the
-// host reads the N_v residual norms once per iteration to apply the rules.
+// Per-RHS coefficients are formed on the device from FP64 reductions.  CG
+// enqueues a run of iterations ahead; the device applies the rule that ends
+// an unconverged run (CgScalars) and the host reads the run's norms once, at
+// its end.  BiCGstab reads them once per iteration.  (8^4, D_S, N_v = 3, FP32:
+// 76 us per iteration with three reductions' second stages, two coefficient
+// kernels and a host read in each, 28 us now; 16^3x32, D_W, N_v = 4: 0.34 and
+// 0.20 ms, where the site-inner order counts too.)
 #include <math.h>
 #include <string.h>
 
@@ -32,11 +37,16 @@ constexpr int kNS = 64;   // max RHS
 struct Ws {
     void *v[kWsVecs];
     double *rr, *rr_new, *pq, *alpha, *beta, *act, *nb, *c1, *c2, *c3, *omega, *rho, *rho_new, *tt;
+    double *rr_prev, *best, *rmax, *since, *sig;
+    double *run;        // [0], [1] the control integers, then kCgHistory x 3 x nv doubles of history
+    double *partial;
+    unsigned *counter;
 };
 
 static int get_ws(const dirac_op *op, Ws &w) {
     dirac_op *self = (dirac_op *)op;
-    const size_t scal = 16 * kNS * 2 * sizeof(double);
+    constexpr int kArrays = 20, kRun = 2 + kCgHistory * 3 * kNS;
+    const size_t scal = (kArrays * kNS * 2 + kRun + 1 + (size_t)kCgBlocks * kNS) * sizeof(double);
     const size_t need = kWsVecs * op->vec_bytes + scal;
     if (!self->solver_ws) {
         if (cudaMalloc(&self->solver_ws, need) != cudaSuccess) {
@@ -46,51 +56,72 @@ static int get_ws(const dirac_op *op, Ws &w) {
         }
         self->solver_ws_bytes = need;
     }
+    if (!self->solver_host &&
+        cudaMallocHost((void **)&self->solver_host, kRun * sizeof(double)) != cudaSuccess) {
+        cudaGetLastError();
+        self->solver_host = nullptr;
+        return DIRAC_ERR_OOM;
+    }
     char *base = (char *)self->solver_ws;
     for (int i = 0; i < kWsVecs; ++i) w.v[i] = base + i * op->vec_bytes;
     double *d = (double *)(base + kWsVecs * op->vec_bytes);
     double **arr[] = {&w.rr, &w.rr_new, &w.pq, &w.alpha, &w.beta, &w.act, &w.nb, &w.c1,
-                      &w.c2, &w.c3, &w.omega, &w.rho, &w.rho_new, &w.tt};
+                      &w.c2, &w.c3, &w.omega, &w.rho, &w.rho_new, &w.tt, &w.rr_prev, &w.best, &w.rmax, &w.since, &w.sig};
+    static_assert(sizeof(arr) / sizeof(arr[0]) <= kArrays, "solver scalars");
     for (size_t i = 0; i < sizeof(arr) / sizeof(arr[0]); ++i) *arr[i] = d + i * kNS * 2;
+    w.run = d + kArrays * kNS * 2;
+    w.counter = (unsigned *)(w.run + kRun);
+    w.partial = w.run + kRun + 1;
     return DIRAC_OK;
 }
 
-// The operator's solver workspace: the first nvecs vectors and the scalar
-// area (arrays of 2*64 doubles in the order rr, rr_new, pq, alpha, beta, act,
-// nb, ...), for drivers in other translation units.
-static int apply_A_pq(const dirac_op *op, const void *p, void *q, double *pq, double m0, cudaStream_t s);
-
-int batch_apply_A_pq(const dirac_op *op, const void *p, void *q, double *pq, double m0, cudaStream_t s) {
-    return apply_A_pq(op, p, q, pq, m0, s);
+static CgScalars cg_scalars(const Ws &w) {
+    CgScalars c{};
+    c.rr = w.rr;
+    c.rr_prev = w.rr_prev;
+    c.pq = w.pq;
+    c.alpha = w.alpha;
+    c.beta = w.beta;
+    c.act = w.act;
+    c.rule = CgScalars::kNone;
+    c.nb = w.nb;
+    c.sig = w.sig;
+    c.best = w.best;
+    c.rmax = w.rmax;
+    c.since = w.since;
+    c.partial = w.partial;
+    c.counter = w.counter;
+    return c;
 }
 
-int solver_ws(const dirac_op *op, void **vecs, int nvecs, double **scal) {
+// The operator's solver workspace for drivers in other translation units: the
+// first nvecs vectors and the CG scalars.
+int solver_cg(const dirac_op *op, void **vecs, int nvecs, CgScalars *c, cudaStream_t s) {
     Ws w;
     int rc = get_ws(op, w);
     if (rc) return rc;
     for (int i = 0; i < nvecs && i < kWsVecs; ++i) vecs[i] = w.v[i];
-    *scal = w.rr;
-    return DIRAC_OK;
+    *c = cg_scalars(w);
+    c->positive = true;
+    return cuda_check(cudaMemsetAsync(w.counter, 0, sizeof(unsigned), s), "reduction counter");
 }
 
 // ---------------------------------------------------------------- coefficient kernels
-// alpha = rr / <p, A p>; pq holds N_v real values <p, D^dag D p> = |D p|^2
-__global__ void cg_alpha_kernel(int nv, const double *rr, const double *pq, const double *act, double *alpha) {
+// beta = rr_new / rr_prev, rr = rr_new (a residual recomputed after the
+// iterated one had already replaced rr)
+__global__ void cg_beta_kernel(int nv, const double *rr_new, CgScalars c) {
     const int v = threadIdx.x;
     if (v >= nv) return;
-    const double p = pq[v];
-    const double a = (act[v] != 0.0 && p != 0.0) ? rr[v] / p : 0.0;
-    alpha[2 * v] = a;
-    alpha[2 * v + 1] = 0.0;
+    const double ro = c.rr_prev[v];
+    const bool on = c.act[v] != 0.0 && (c.positive ? ro > 0.0 : ro != 0.0);
+    c.beta[2 * v] = on ? rr_new[v] / ro : 0.0;
+    c.beta[2 * v + 1] = 0.0;
+    c.rr[v] = rr_new[v];
 }
 
-__global__ void cg_beta_kernel(int nv, const double *rr_new, double *rr, const double *act, double *beta) {
-    const int v = threadIdx.x;
-    if (v >= nv) return;
-    const double b = (act[v] != 0.0 && rr[v] != 0.0) ? rr_new[v] / rr[v] : 0.0;
-    beta[2 * v] = b;
-    beta[2 * v + 1] = 0.0;
-    rr[v] = rr_new[v];
+int solver_cg_beta(const dirac_op *op, const double *rr_new, const CgScalars &c, cudaStream_t s) {
+    cg_beta_kernel<<<1, kNS, 0, s>>>(op->nv, rr_new, c);
+    return launch_check("cg_beta_kernel");
 }
 
 __device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
@@ -255,17 +286,107 @@ static int apply_A(const dirac_op *op, const void *in, void *out, double m0, cud
     return op_apply_cg(op, in, out, m0, s);
 }
 
-// q = D^dag D p through the operator scratch, with pq = Re <p, q> per RHS.
+// q = D^dag D p through the operator scratch, then pq = Re <p, q> and alpha.
 // The step length must match the q that is subtracted from r: |D p|^2 from
 // the intermediate would save one vector read, but it differs from <p, q> by
 // the rounding of D p and of q, and in FP32 the gap between the updated and
 // the true residual then grows until the 1% rule stops the solve (measured on
 // staggered solves at cond ~ 2e3).
-static int apply_A_pq(const dirac_op *op, const void *p, void *q, double *pq, double m0, cudaStream_t s) {
-    int rc = op_apply(op, p, is_laplace(op->kind) ? q : op->scratch, m0, +1, s);
-    if (!rc && !is_laplace(op->kind)) rc = op_apply(op, op->scratch, q, m0, -1, s);
-    if (!rc) rc = blas_dot_re(op, op->prec, p, q, pq, s);
-    return rc;
+int solver_cg_step(const dirac_op *op, const void *p, void *q, double m0, const CgScalars &c, cudaStream_t s) {
+    int rc = op_apply_cg(op, p, q, m0, s);
+    return rc ? rc : blas_cg_dot(op, op->prec, p, q, c, s);
+}
+
+// A run of CG iterations enqueued ahead, as the host sees it afterwards.
+struct CgRun {
+    int done = 0;                  // iterations the device carried out
+    const double *hist = nullptr;  // done x (pq, old rr, new rr) x nv
+    double log_rate = -0.5;        // last seen change of log |r|^2 per iteration (slowest RHS)
+};
+
+// Largest vector whose iterations go through a graph: above it an iteration
+// takes long enough for the stream to keep up.
+constexpr size_t kCgGraphBytes = 32u << 20;
+
+// How many iterations to enqueue before the host looks again.  The launches of
+// iterations past the stop rule cost little (their vector passes return at
+// once) but their stencils run, so the run stays short of where the residual
+// is predicted to pass: `need` = log of the drop in |r|^2 still missing.
+static int run_length(const CgRun &run, double need) {
+    double n = need / run.log_rate;   // both negative
+    if (!(n > 0)) n = 1;
+    n *= 0.7;
+    return n < 1 ? 1 : n > kCgHistory ? kCgHistory : (int)n;
+}
+
+// The launches of one iteration: the update of x and p that the one before
+// left due, q = A p with alpha, and r with beta.
+static int cg_iteration(const dirac_op *op, void *r, void *pv, void *q, void *x, double m0, const CgScalars &c,
+                        cudaStream_t s) {
+    TRY(blas_cg_update(op, op->prec, x, pv, r, c, s));
+    TRY(solver_cg_step(op, pv, q, m0, c, s));
+    return blas_cg_residual(op, op->prec, r, q, c, s);
+}
+
+// kUnroll iterations as a CUDA graph, for one solve: on small lattices the
+// launches of a stream follow one another no faster than about every 4 us,
+// the nodes of a graph every 2 us.
+struct CgGraph {
+    static constexpr int kUnroll = 5;   // divides the usual recompute intervals (20, 50)
+    cudaGraphExec_t exec = nullptr;
+    bool tried = false;
+    CgGraph() = default;
+    CgGraph(const CgGraph &) = delete;
+    CgGraph &operator=(const CgGraph &) = delete;
+    ~CgGraph() {
+        if (exec) cudaGraphExecDestroy(exec);
+    }
+    // Record the iterations on a stream of our own (the caller's may be the
+    // legacy default stream, which cannot be captured).  Without a graph the
+    // solve launches them one by one.
+    template <typename F>
+    void build(F &&iteration) {
+        tried = true;
+        cudaStream_t cap = nullptr;
+        cudaGraph_t g = nullptr;
+        bool ok = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) == cudaSuccess &&
+                  cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+        if (ok) {
+            for (int k = 0; k < kUnroll && ok; ++k) ok = iteration(cap) == DIRAC_OK;
+            ok = cudaStreamEndCapture(cap, &g) == cudaSuccess && ok;
+            if (ok && cudaGraphInstantiate(&exec, g, 0) != cudaSuccess) exec = nullptr;
+        }
+        if (g) cudaGraphDestroy(g);
+        if (cap) cudaStreamDestroy(cap);
+        cudaGetLastError();
+    }
+};
+
+// Enqueue n iterations of r, q, p (x or the accumulated correction y) and wait
+// for them.  After it, the last iteration's residual is updated and its update
+// of x and p is due.
+static int cg_run(const dirac_op *op, void *r, void *pv, void *q, void *x, double m0, int n, const CgScalars &c, Ws &w,
+                  CgRun &run, CgGraph &graph, cudaStream_t s) {
+    const int nv = op->nv;
+    TRY(cuda_check(cudaMemsetAsync(w.run, 0, sizeof(double), s), "run control"));
+    auto iteration = [&](cudaStream_t t) { return cg_iteration(op, r, pv, q, x, m0, c, t); };
+    if (n >= CgGraph::kUnroll && !graph.tried && op->vec_bytes <= kCgGraphBytes) graph.build(iteration);
+    int k = 0;
+    if (graph.exec)
+        for (; k + CgGraph::kUnroll <= n; k += CgGraph::kUnroll)
+            TRY(cuda_check(cudaGraphLaunch(graph.exec, s), "cg graph"));
+    for (; k < n; ++k) TRY(iteration(s));
+    TRY(to_host(op->solver_host, w.run, 2 + n * 3 * nv, s));
+    run.done = ((const int *)op->solver_host)[1];
+    run.hist = op->solver_host + 2;
+    if (run.done < 1 || run.done > n) return DIRAC_ERR_CUDA;   // the launches did not run
+    double rate = -1e300;
+    for (int v = 0; v < nv; ++v) {
+        const double first = run.hist[nv + v], last = run.hist[((run.done - 1) * 3 + 2) * nv + v];
+        if (first > 0 && last > 0) rate = fmax(rate, log(last / first) / run.done);
+    }
+    if (rate > -1e300 && rate < -1e-3) run.log_rate = rate;
+    return DIRAC_OK;
 }
 
 // CG on A x = rhs (A = D^dag D), x in/out.  Uses ws vectors 0..2.
@@ -277,68 +398,85 @@ static int cg_core(const dirac_op *op, const void *rhs, void *x, double m0, doub
     const dirac_prec p = op->prec;
     void *r = w.v[0], *pv = w.v[1], *q = w.v[2];
     double nb[kNS], rr[kNS], act[kNS], rrt[kNS];
+    TRY(cuda_check(cudaMemsetAsync(w.counter, 0, sizeof(unsigned), s), "reduction counter"));
     TRY(blas_norm2(op, p, rhs, w.nb, s));
-    TRY(to_host(nb, w.nb, nv, s));
     // r = rhs - A x
     TRY(apply_A(op, x, q, m0, s));
     TRY(blas_axpby(op, p, r, rhs, nullptr, 1.0, q, nullptr, -1.0, w.rr, s));
     TRY(blas_axpby(op, p, pv, r, nullptr, 1.0, nullptr, nullptr, 0.0, nullptr, s));
+    TRY(to_host(nb, w.nb, nv, s));
     TRY(to_host(rr, w.rr, nv, s));
     int nact = 0;
+    double need = 0;
     for (int v = 0; v < nv; ++v) {
         const bool conv = nb[v] == 0.0 || sqrt(rr[v]) < tol * sqrt(nb[v]);
         act[v] = conv ? 0.0 : 1.0;
         out.status_rhs[v] = conv ? DIRAC_OK : DIRAC_NOT_CONVERGED;
         out.relres[v] = nb[v] > 0 ? sqrt(rr[v] / nb[v]) : 0.0;
         nact += !conv;
+        if (!conv) need = fmin(need, log(tol * tol * nb[v] / rr[v]));
     }
     TRY(to_dev(w.act, act, nv, s));
+    CgScalars c = cg_scalars(w);
+    c.rule = CgScalars::kPlain;
+    c.tol = tol;
+    c.ctl = (int *)w.run;
+    c.hist = w.run + 2;
+    CgRun run;
+    CgGraph graph;
+    TRY(cuda_check(cudaMemsetAsync(w.run, 0, 2 * sizeof(double), s), "run control"));
     out.status = DIRAC_OK;
     int it = 0;
     while (nact > 0) {
-        ++it;
-        TRY(apply_A_pq(op, pv, q, w.pq, m0, s));
-        cg_alpha_kernel<<<1, kNS, 0, s>>>(nv, w.rr, w.pq, w.act, w.alpha);
-        TRY(blas_axpby(op, p, r, r, nullptr, 1.0, q, w.alpha, -1.0, w.rr_new, s));
-        double rn[kNS], pq[kNS], rro[kNS];
-        if (lan) {
-            TRY(cuda_check(cudaMemcpyAsync(pq, w.pq, nv * sizeof(double), cudaMemcpyDeviceToHost, s), "D2H"));
-            TRY(cuda_check(cudaMemcpyAsync(rro, w.rr, nv * sizeof(double), cudaMemcpyDeviceToHost, s), "D2H"));
-        }
-        TRY(to_host(rn, w.rr_new, nv, s));
-        if (lan) lan->add(nv, act, rro, pq, rn);
+        int n = run_length(run, need);
+        if (it == 0 && n > 4) n = 4;   // no rate seen yet
+        n = n < every - it % every ? n : every - it % every;
+        n = n < maxit - it ? n : maxit - it;
+        TRY(cg_run(op, r, pv, q, x, m0, n, c, w, run, graph, s));
+        if (lan)
+            for (int k = 0; k < run.done; ++k) {
+                const double *h = run.hist + k * 3 * nv;
+                lan->add(nv, act, h + nv, h, h + 2 * nv);
+            }
+        it += run.done;
+        const double *rn = run.hist + ((run.done - 1) * 3 + 2) * nv;
         bool all_pass = true, finite = true;
+        need = 0;
         for (int v = 0; v < nv; ++v) {
             if (!isfinite(rn[v])) finite = false;
-            if (act[v] != 0.0 && !(sqrt(rn[v]) < tol * sqrt(nb[v]))) all_pass = false;
+            if (act[v] != 0.0 && !(sqrt(rn[v]) < tol * sqrt(nb[v]))) {
+                all_pass = false;
+                need = fmin(need, log(tol * tol * nb[v] / rn[v]));
+            }
         }
         if (!finite) {
             out.status = DIRAC_NONFINITE;
             break;
         }
-        const bool recompute = it % every == 0 || all_pass || it >= maxit;
-        if (recompute) {
-            // the solution update is needed now; otherwise it is fused with p below
+        if (it % every == 0 || all_pass || it >= maxit) {
             TRY(blas_axpby(op, p, x, x, nullptr, 1.0, pv, w.alpha, 1.0, nullptr, s));
             out.recomputes++;
             TRY(apply_A(op, x, q, m0, s));
             TRY(blas_axpby(op, p, r, rhs, nullptr, 1.0, q, nullptr, -1.0, w.rr_new, s));
             TRY(to_host(rrt, w.rr_new, nv, s));
-            bool stagnated = false;
+            bool stagnated = false, froze = false;
             nact = 0;
+            need = 0;
             for (int v = 0; v < nv; ++v) {
                 out.relres[v] = nb[v] > 0 ? sqrt(rrt[v] / nb[v]) : 0.0;
                 if (act[v] == 0.0) continue;
                 if (sqrt(rrt[v]) < tol * sqrt(nb[v])) {
                     act[v] = 0.0;
+                    froze = true;
                     out.status_rhs[v] = DIRAC_OK;
                     continue;
                 }
                 const double disc = fabs(sqrt(rn[v]) - sqrt(rrt[v])) / fmax(sqrt(rrt[v]), 1e-300);
                 if (disc > 0.01) stagnated = true;
+                need = fmin(need, log(tol * tol * nb[v] / rrt[v]));
                 ++nact;
             }
-            TRY(to_dev(w.act, act, nv, s));
+            if (froze) TRY(to_dev(w.act, act, nv, s));
             if (nact == 0) break;
             if (stagnated) {
                 out.status = DIRAC_STAGNATED;
@@ -350,10 +488,10 @@ static int cg_core(const dirac_op *op, const void *rhs, void *x, double m0, doub
                 out.status = DIRAC_NOT_CONVERGED;
                 break;
             }
+            TRY(solver_cg_beta(op, w.rr_new, c, s));
+            TRY(blas_axpby(op, p, pv, r, nullptr, 1.0, pv, w.beta, 1.0, nullptr, s));
+            TRY(cuda_check(cudaMemsetAsync(w.run, 0, 2 * sizeof(double), s), "run control"));   // nothing due
         }
-        cg_beta_kernel<<<1, kNS, 0, s>>>(nv, w.rr_new, w.rr, w.act, w.beta);
-        if (recompute) TRY(blas_axpby(op, p, pv, r, nullptr, 1.0, pv, w.beta, 1.0, nullptr, s));
-        else TRY(blas_update_xp(op, p, x, pv, r, w.alpha, w.beta, s));   // x += alpha p; p = r + beta p
     }
     out.iters = it;
     TRY(launch_check("cg coefficient kernels"));
@@ -508,6 +646,7 @@ static int cg_reliable(const dirac_op *hi, const dirac_op *lo, const void *rhs, 
     void *rh = wh.v[0], *th = wh.v[1];
     void *rs = wl.v[0], *ps = wl.v[1], *qs = wl.v[2], *ys = wl.v[3];
     double *sig = wh.c1, *ratio = wh.c3, *inv = wh.omega;
+    TRY(cuda_check(cudaMemsetAsync(wl.counter, 0, sizeof(unsigned), s), "reduction counter"));
     double nb[kNS], rrt[kNS], act[kNS], rmax[kNS], prev_true[kNS], best[kNS], best_true[kNS];
     int slow[kNS], since_best[kNS];
     // sloppy iterations without a new residual minimum that force an update
@@ -537,7 +676,7 @@ static int cg_reliable(const dirac_op *hi, const dirac_op *lo, const void *rhs, 
     const double unit = sqrt((double)hi->rows);
     coef_from_norm_kernel<<<1, kNS, 0, s>>>(nv, wh.rr, wh.act, sig, 1, unit);
     TRY(blas_axpby(hi, ph, th, rh, sig, 1.0, nullptr, nullptr, 0.0, nullptr, s));
-    TRY(blas_convert(hi, th, ph, rs, pl, s));
+    TRY(blas_convert_layout(hi, th, ph, hi->geom.layout, rs, pl, lo->geom.layout, s));
     TRY(blas_axpby(lo, pl, ps, rs, nullptr, 1.0, nullptr, nullptr, 0.0, nullptr, s));
     TRY(cuda_check(cudaMemsetAsync(ys, 0, lo->vec_bytes, s), "memset"));
     TRY(blas_norm2(lo, pl, rs, wl.rr, s));
@@ -549,34 +688,67 @@ static int cg_reliable(const dirac_op *hi, const dirac_op *lo, const void *rhs, 
     }
     double sig_h[kNS];
     for (int v = 0; v < nv; ++v) sig_h[v] = (act[v] != 0.0 && rrt[v] > 0) ? unit / sqrt(rrt[v]) : 0.0;
+    // the device's copies of what decides a refresh
+    double goal[kNS];   // log of |r|^2 at the refresh each RHS is heading for
+    auto upload = [&]() -> int {
+        double zero[kNS] = {};
+        for (int v = 0; v < nv; ++v)
+            goal[v] = 2 * log(fmax(fmax(delta * rmax[v], tol * sqrt(nb[v]) * sig_h[v]), 1e-300));
+        TRY(to_dev(wl.nb, nb, nv, s));
+        TRY(to_dev(wl.sig, sig_h, nv, s));
+        TRY(to_dev(wl.best, best, nv, s));
+        TRY(to_dev(wl.rmax, rmax, nv, s));
+        return to_dev(wl.since, zero, nv, s);
+    };
+    TRY(upload());
+    CgScalars c = cg_scalars(wl);
+    c.rule = CgScalars::kReliable;
+    c.tol = tol;
+    c.delta = delta;
+    c.stall = kStall;
+    c.ctl = (int *)wl.run;
+    c.hist = wl.run + 2;
+    CgRun run;
+    CgGraph graph;
+    TRY(cuda_check(cudaMemsetAsync(wl.run, 0, 2 * sizeof(double), s), "run control"));
+    double need = -1;
     out.status = DIRAC_OK;
     int it = 0;
     while (nact > 0) {
-        ++it;
-        TRY(apply_A_pq(lo, ps, qs, wl.pq, m0, s));
-        cg_alpha_kernel<<<1, kNS, 0, s>>>(nv, wl.rr, wl.pq, wl.act, wl.alpha);
-        TRY(blas_axpby(lo, pl, rs, rs, nullptr, 1.0, qs, wl.alpha, -1.0, wl.rr_new, s));
-        double rn[kNS], pq[kNS], rro[kNS];
-        if (lan) {
-            TRY(cuda_check(cudaMemcpyAsync(pq, wl.pq, nv * sizeof(double), cudaMemcpyDeviceToHost, s), "D2H"));
-            TRY(cuda_check(cudaMemcpyAsync(rro, wl.rr, nv * sizeof(double), cudaMemcpyDeviceToHost, s), "D2H"));
-        }
-        TRY(to_host(rn, wl.rr_new, nv, s));
-        if (lan) lan->add(nv, act, rro, pq, rn);
-        bool trigger = it >= maxit, finite = true;
+        int n = run_length(run, need);
+        if (it == 0 && n > 4) n = 4;   // no rate seen yet
+        n = n < maxit - it ? n : maxit - it;
+        TRY(cg_run(lo, rs, ps, qs, ys, m0, n, c, wl, run, graph, s));
+        bool trigger = false, finite = true;
         bool stalled[kNS];
-        for (int v = 0; v < nv; ++v) {
-            stalled[v] = false;
-            if (!isfinite(rn[v])) finite = false;
-            if (act[v] == 0.0) continue;
-            const double r = sqrt(rn[v]);
-            if (r < best[v]) {
-                best[v] = r;
-                since_best[v] = 0;
-            } else if (++since_best[v] >= kStall) {
-                trigger = true;   // the sloppy recurrence stopped improving: refresh it
+        const double *rn_dev = nullptr;
+        for (int k = 0; k < run.done; ++k) {   // the device's rule over again, for the host's copies
+            const double *h = run.hist + k * 3 * nv;
+            const double *rk = rn_dev = h + 2 * nv;
+            ++it;
+            if (lan) lan->add(nv, act, h + nv, h, rk);
+            trigger = it >= maxit;
+            for (int v = 0; v < nv; ++v) {
+                stalled[v] = false;
+                if (!isfinite(rk[v])) finite = false;
+                if (act[v] == 0.0) continue;
+                const double r = sqrt(rk[v]);
+                if (r < best[v]) {
+                    best[v] = r;
+                    since_best[v] = 0;
+                } else if (++since_best[v] >= kStall) {
+                    trigger = true;   // the sloppy recurrence stopped improving: refresh it
+                }
+                if (r < delta * rmax[v] || r < tol * sqrt(nb[v]) * sig_h[v]) trigger = true;
             }
-            if (r < delta * rmax[v] || r < tol * sqrt(nb[v]) * sig_h[v]) trigger = true;
+            if (!trigger)
+                for (int v = 0; v < nv; ++v) rmax[v] = fmax(rmax[v], sqrt(rk[v]));
+        }
+        double rn[kNS];
+        need = -1e300;
+        for (int v = 0; v < nv; ++v) {
+            rn[v] = rn_dev[v];
+            if (act[v] != 0.0 && rn[v] > 0) need = fmax(need, goal[v] - log(rn[v]));
         }
         if (!finite) {
             out.status = DIRAC_NONFINITE;
@@ -587,7 +759,7 @@ static int cg_reliable(const dirac_op *hi, const dirac_op *lo, const void *rhs, 
             TRY(blas_axpby(lo, pl, ys, ys, nullptr, 1.0, ps, wl.alpha, 1.0, nullptr, s));
             // x += y / sigma, then the true residual in the high precision
             inverse_kernel<<<1, kNS, 0, s>>>(nv, sig, inv);
-            TRY(blas_convert(lo, ys, pl, th, ph, s));
+            TRY(blas_convert_layout(lo, ys, pl, lo->geom.layout, th, ph, hi->geom.layout, s));
             TRY(blas_axpby(hi, ph, x, x, nullptr, 1.0, th, inv, 1.0, nullptr, s));
             TRY(apply_A(hi, x, th, m0, s));
             TRY(blas_axpby(hi, ph, rh, rhs, nullptr, 1.0, th, nullptr, -1.0, wh.rr, s));
@@ -642,9 +814,9 @@ static int cg_reliable(const dirac_op *hi, const dirac_op *lo, const void *rhs, 
             }
             TRY(to_dev(ratio, rat, 2 * nv, s));
             coef_from_norm_kernel<<<1, kNS, 0, s>>>(nv, wh.rr, wh.act, sig, 1, unit);
-            scale_rr_kernel<<<1, kNS, 0, s>>>(nv, ratio, wl.rr);
+            scale_rr_kernel<<<1, kNS, 0, s>>>(nv, ratio, wl.rr_prev);
             TRY(blas_axpby(hi, ph, th, rh, sig, 1.0, nullptr, nullptr, 0.0, nullptr, s));
-            TRY(blas_convert(hi, th, ph, rs, pl, s));
+            TRY(blas_convert_layout(hi, th, ph, hi->geom.layout, rs, pl, lo->geom.layout, s));
             TRY(blas_axpby(lo, pl, ps, ps, ratio, 1.0, nullptr, nullptr, 0.0, nullptr, s));
             TRY(cuda_check(cudaMemsetAsync(ys, 0, lo->vec_bytes, s), "memset"));
             TRY(blas_norm2(lo, pl, rs, wl.rr_new, s));
@@ -654,12 +826,14 @@ static int cg_reliable(const dirac_op *hi, const dirac_op *lo, const void *rhs, 
                 since_best[v] = 0;
                 sig_h[v] = (act[v] != 0.0 && rrt[v] > 0) ? unit / sqrt(rrt[v]) : 0.0;
             }
-        } else {
-            for (int v = 0; v < nv; ++v) rmax[v] = fmax(rmax[v], sqrt(rn[v]));
+            TRY(upload());
+            need = -1e300;
+            for (int v = 0; v < nv; ++v)
+                if (act[v] != 0.0 && rn[v] > 0) need = fmax(need, goal[v] - log(rn[v]));
+            TRY(solver_cg_beta(lo, wl.rr_new, c, s));
+            TRY(blas_axpby(lo, pl, ps, rs, nullptr, 1.0, ps, wl.beta, 1.0, nullptr, s));
+            TRY(cuda_check(cudaMemsetAsync(wl.run, 0, 2 * sizeof(double), s), "run control"));   // nothing due
         }
-        cg_beta_kernel<<<1, kNS, 0, s>>>(nv, wl.rr_new, wl.rr, wl.act, wl.beta);
-        if (trigger) TRY(blas_axpby(lo, pl, ps, rs, nullptr, 1.0, ps, wl.beta, 1.0, nullptr, s));
-        else TRY(blas_update_xp(lo, pl, ys, ps, rs, wl.alpha, wl.beta, s));   // y += alpha p; p = r + beta p
     }
     out.iters = it;
     TRY(launch_check("reliable-update kernels"));
@@ -729,7 +903,7 @@ static int mixed_solve(const dirac_op *op, const void *b, void *x, double m0, co
         const double unit = sqrt((double)op->rows);   // unit rms per component (see cg_reliable)
         coef_from_norm_kernel<<<1, kNS, 0, s>>>(nv, wh.rr, wh.act, wh.c1, 1, unit);
         TRY(blas_axpby(op, ph, tmp, r, wh.c1, 1.0, nullptr, nullptr, 0.0, nullptr, s));
-        TRY(blas_convert(op, tmp, ph, rl, pl, s));
+        TRY(blas_convert_layout(op, tmp, ph, op->geom.layout, rl, pl, lo->geom.layout, s));
         TRY(cuda_check(cudaMemsetAsync(el, 0, lo->vec_bytes, s), "memset"));
         CoreOut co;
         const int budget = prm->maxit - total;
@@ -738,7 +912,7 @@ static int mixed_solve(const dirac_op *op, const void *b, void *x, double m0, co
         total += co.iters;
         st->recomputes += co.recomputes;
         // x += |r| e
-        TRY(blas_convert(op, el, pl, tmp, ph, s));
+        TRY(blas_convert_layout(op, el, pl, lo->geom.layout, tmp, ph, op->geom.layout, s));
         coef_from_norm_kernel<<<1, kNS, 0, s>>>(nv, wh.rr, wh.act, wh.c1, 0, unit);
         TRY(blas_axpby(op, ph, x, x, nullptr, 1.0, tmp, wh.c1, 1.0, nullptr, s));
         ++outer;
@@ -811,17 +985,31 @@ static int plain_solve(const dirac_op *op, const void *b, void *x, double m0, co
     const int every = prm->recompute_every > 0 ? prm->recompute_every : (op->prec == DIRAC_F64 ? 50 : 20);
     CoreOut co;
     Lanczos lan;
+    // the iteration runs on site-inner vectors: b and x of a site-outer
+    // operator are reordered once each way (ws vectors 5 to 7 are free here)
+    const int lay = op->geom.layout;
+    const bool reorder = lay != DIRAC_LAYOUT_SITE_INNER;
+    const dirac_op view = op_site_inner(op);
+    const void *bi = b;
+    void *xi = x;
+    if (reorder) {
+        TRY(blas_convert_layout(op, b, op->prec, lay, w.v[6], op->prec, DIRAC_LAYOUT_SITE_INNER, s));
+        TRY(blas_convert_layout(op, x, op->prec, lay, w.v[7], op->prec, DIRAC_LAYOUT_SITE_INNER, s));
+        bi = w.v[6];
+        xi = w.v[7];
+    }
     if (prm->solver == DIRAC_CG_NORMAL) {
         void *rhs = w.v[5];
-        TRY(op_apply(op, b, rhs, m0, -1, s));
-        TRY(cg_core(op, rhs, x, m0, prm->tol, prm->maxit, every, co, s, &lan));
+        TRY(op_apply(&view, bi, rhs, m0, -1, s));
+        TRY(cg_core(&view, rhs, xi, m0, prm->tol, prm->maxit, every, co, s, &lan));
         lanczos_stats(lan, op->nv, st);
     } else if (prm->solver == DIRAC_CG_HPD) {
-        TRY(cg_core(op, b, x, m0, prm->tol, prm->maxit, every, co, s, &lan));
+        TRY(cg_core(&view, bi, xi, m0, prm->tol, prm->maxit, every, co, s, &lan));
         lanczos_stats(lan, op->nv, st);
     } else {
-        TRY(bicgstab_core(op, b, x, m0, prm->tol, prm->maxit, every, co, s));
+        TRY(bicgstab_core(&view, bi, xi, m0, prm->tol, prm->maxit, every, co, s));
     }
+    if (reorder) TRY(blas_convert_layout(op, xi, op->prec, DIRAC_LAYOUT_SITE_INNER, x, op->prec, lay, s));
     st->iters = co.iters;
     st->outer_iters = 0;
     st->recomputes = co.recomputes;
