@@ -451,6 +451,7 @@ template <typename E, int LAYOUT, typename EL>
 int launch_brillouin_v(const dirac_op *op, const void *in, void *out, double m0, int sgn, cudaStream_t s) {
     int vr, minb, block;
     launch_variant(op, vr, minb, block);
+    vr = aligned_vr(vr, op->prec, in, out);
     using A = typename Acc<E>::T;
     return dispatch_nc<big_nc_ok<E>()>(op->nc, [&](auto ncc) {
         constexpr int NC = decltype(ncc)::value;

@@ -131,6 +131,14 @@ struct Prod<float, true> {
     static __device__ __forceinline__ Vec scale(float f, const Vec &v) { return mul2(bcast2(f), v); }
 };
 
+// a, or -a where neg: on the integer pipe (an FP64 multiply by -1 is slow)
+__device__ __forceinline__ float flip(float a, bool neg) { return __int_as_float(__float_as_int(a) ^ (neg ? 0x80000000 : 0)); }
+__device__ __forceinline__ double flip(double a, bool neg) {
+    return __hiloint2double(__double2hiint(a) ^ (neg ? 0x80000000 : 0), __double2loint(a));
+}
+template <typename A>
+__device__ __forceinline__ cx<A> flip(cx<A> a, bool neg) { return cx<A>{flip(a.re, neg), flip(a.im, neg)}; }
+
 // -------------------------------------------------------- storage elements
 template <typename E> struct Acc { using T = float; };
 template <> struct Acc<double> { using T = double; };
@@ -157,21 +165,41 @@ template <> struct Raw<16> { using T = uint4; };
 template <> struct Raw<8> { using T = uint2; };
 template <> struct Raw<4> { using T = unsigned int; };
 
+// 32-byte global accesses (one instruction, four sectors of a line per two
+// lanes): a lane that takes 32 consecutive bytes as two 16-byte loads makes
+// either load touch twice the lines it needs.
+__device__ __forceinline__ void ld32(const void *p, unsigned (&r)[8]) {
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+        : "l"(p));
+}
+__device__ __forceinline__ void st32(void *p, const unsigned (&r)[8]) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(r[0]), "r"(r[1]), "r"(r[2]),
+                 "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+                 : "memory");
+}
+
 // Load N consecutive complex numbers starting at element pointer p (2N
-// elements), converting to the accumulation type.  Uses 16-byte (or smaller)
-// vector loads; p must be aligned to min(16, 2*N*sizeof(E)) bytes.
+// elements), converting to the accumulation type.  Uses one vector load of at
+// most 32 bytes; p must be aligned to min(32, 2*N*sizeof(E)) bytes.
 template <typename E, int N, typename A = typename Acc<E>::T>
 __device__ __forceinline__ void load_cx(const E *__restrict__ p, cx<A> *out) {
     constexpr int BYTES = 2 * N * (int)sizeof(E);
-    if constexpr (BYTES <= 16) {
-        using R = typename Raw<BYTES>::T;
-        R raw = __ldg(reinterpret_cast<const R *>(p));
+    if constexpr (BYTES <= 32) {
         E e[2 * N];
-        __builtin_memcpy(e, &raw, BYTES);
+        if constexpr (BYTES == 32) {
+            unsigned raw[8];
+            ld32(p, raw);
+            __builtin_memcpy(e, raw, BYTES);
+        } else {
+            using R = typename Raw<BYTES>::T;
+            R raw = __ldg(reinterpret_cast<const R *>(p));
+            __builtin_memcpy(e, &raw, BYTES);
+        }
 #pragma unroll
         for (int i = 0; i < N; ++i) out[i] = cx<A>{(A)to_acc<E>(e[2 * i]), (A)to_acc<E>(e[2 * i + 1])};
     } else {
-        constexpr int PER = 16 / (2 * (int)sizeof(E));
+        constexpr int PER = 32 / (2 * (int)sizeof(E));
 #pragma unroll
         for (int k = 0; k < N / PER; ++k) load_cx<E, PER, A>(p + 2 * PER * k, out + PER * k);
     }
@@ -180,19 +208,25 @@ __device__ __forceinline__ void load_cx(const E *__restrict__ p, cx<A> *out) {
 template <typename E, int N, typename A>
 __device__ __forceinline__ void store_cx(E *__restrict__ p, const cx<A> *in) {
     constexpr int BYTES = 2 * N * (int)sizeof(E);
-    if constexpr (BYTES <= 16) {
-        using R = typename Raw<BYTES>::T;
+    if constexpr (BYTES <= 32) {
         E e[2 * N];
 #pragma unroll
         for (int i = 0; i < N; ++i) {
             e[2 * i] = from_acc<E, A>(in[i].re);
             e[2 * i + 1] = from_acc<E, A>(in[i].im);
         }
-        R raw;
-        __builtin_memcpy(&raw, e, BYTES);
-        *reinterpret_cast<R *>(p) = raw;
+        if constexpr (BYTES == 32) {
+            unsigned raw[8];
+            __builtin_memcpy(raw, e, BYTES);
+            st32(p, raw);
+        } else {
+            using R = typename Raw<BYTES>::T;
+            R raw;
+            __builtin_memcpy(&raw, e, BYTES);
+            *reinterpret_cast<R *>(p) = raw;
+        }
     } else {
-        constexpr int PER = 16 / (2 * (int)sizeof(E));
+        constexpr int PER = 32 / (2 * (int)sizeof(E));
 #pragma unroll
         for (int k = 0; k < N / PER; ++k) store_cx<E, PER, A>(p + 2 * PER * k, in + PER * k);
     }

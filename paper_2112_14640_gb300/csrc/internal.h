@@ -96,6 +96,7 @@ int dispatch_prec(dirac_prec p, F &&f) {
 // per thread and the compiler's own register choice (kMaxNcSmall below).
 constexpr int kMaxNc = 8;
 constexpr int kMaxNcSmall = 4;
+constexpr int kTunedNc = 3;
 // Products of a stencil over the Brillouin offsets: packed FP32 pairs
 // (common.cuh) where the two accumulators of each of the NC NS VR components
 // leave the register class (the cap of MINB, below) about 60
@@ -166,6 +167,27 @@ inline bool variant_ok(const dirac_op *op, int vr, int minb) {
     return variant_compiled(op->nc, vr, minb) && op->nv % vr == 0;
 }
 
+// Second launch bound of a stencil.  N_c = 3 has its register classes (MINB);
+// the other N_c are compiled once, and there the compiler left to itself often
+// holds few loads in flight (D_W at N_c = 4, VR = 1: 86 registers, 0.525 ms at
+// 16^3x32, N_v = 24; 128 registers: 0.328 ms).  Where it measured faster
+// (`bound`) they get the registers for what a thread keeps: NC NS VR
+// accumulators, `extra` further complex numbers (neighbour components, the
+// link), and about 40 for addresses.  16^4, N_v = 12, FP32, without and with:
+// D_W N_c = 2: 39 and 35 us, 4: 103 and 85 (N_c = 1: 14.9 and 16.0, N_c = 6,
+// N_v = 5: 109 and 117, left alone); D_S N_c = 2: 14 and 12, 4: 35 and 29, 6:
+// 119 and 111 (N_c = 1: 9.7 and 12.3); the Laplacian wlap N_c = 2: 39 and 36
+// (N_c = 4, VR = 1: 102 and 113), blap N_c = 4: 125 and 118 on 8^3x16, 6: 448
+// and 318 (N_c = 2: 47 and 49).
+template <int NC, int NS, int VR, int MINB, typename A>
+constexpr int stencil_min_blocks(bool bound, int extra) {
+    if (MINB > 1) return 1;
+    if (NC == kTunedNc || !bound) return 0;
+    const int need = 2 * (NC * NS * VR + extra) * (int)(sizeof(A) / 4) + 40;
+    const int b = 65536 / (128 * need);
+    return b < 1 ? 1 : b > 8 ? 8 : b;
+}
+
 template <typename F>
 int dispatch_layout(int layout, F &&f) {
     switch (layout) {
@@ -211,12 +233,13 @@ inline void launch_variant(const dirac_op *op, int &vr, int &minb, int &block) {
     vr = op->nc > kMaxNcSmall ? 1 : pick_vr(op->prec, op->nv);
     minb = 1;
     block = kStencilBlock;
+    // D_S reads 24 N_v bytes a site beside 72 of links per hop: the widest
+    // group of one 32-byte access spreads a link over the most RHS (16^3x32,
+    // N_v = 12, FP32: 36 us, two RHS per thread 41 us)
+    if (op->kind == DIRAC_STAGGERED && op->prec == DIRAC_F32 && op->nc <= kMaxNcSmall && op->nv % 4 == 0) vr = 4;
     if (op->nc == 3) {
-        if (op->kind == DIRAC_WILSON) {
-            minb = vr == 4 ? 3 : 4;
-        } else if (op->kind == DIRAC_STAGGERED) {
-            minb = 3;
-        }
+        if (op->kind == DIRAC_WILSON) minb = vr == 4 ? 3 : 4;
+        else if (op->kind == DIRAC_STAGGERED) minb = vr == 4 ? 5 : 6;
     }
     // 81-point stencils on 4 spins in FP32 arithmetic: two accumulators per
     // component (common.cuh), so one RHS per thread from N_c = 3 on (16^3x32,
@@ -226,6 +249,14 @@ inline void launch_variant(const dirac_op *op, int &vr, int &minb, int &block) {
         vr = op->nc >= 3 || vr == 1 ? 1 : 2;
         if (op->nc == 3) minb = 4;
     }
+}
+
+// VR complex numbers of an element are one access of up to 32 bytes, which
+// needs that alignment; vectors are only required to be 16-byte aligned, so a
+// launch on less aligned ones takes the widest group of 16 bytes instead.
+inline int aligned_vr(int vr, dirac_prec p, const void *in, const void *out) {
+    const int most = (int)(16 / (2 * elem_bytes(p)));
+    return vr > most && (((uintptr_t)in | (uintptr_t)out) & 31) ? most : vr;
 }
 
 inline unsigned grid_for(long long threads, int block) {

@@ -102,7 +102,8 @@ __device__ __forceinline__ void lap_write(const E *__restrict__ in, E *__restric
 
 // Eq. (app_wlap): centre = 4 + m^2/2, each hop weighted -1/2
 template <int NC, int NS, int VR, typename E, int MINB, int LAYOUT>
-__global__ void __launch_bounds__(stencil_max_threads(MINB), (MINB > 1 ? 1 : 0))
+__global__ void __launch_bounds__(stencil_max_threads(MINB),
+                                  (stencil_min_blocks<NC, NS, VR, MINB, typename Acc<E>::T>(NC <= 2, NC * NS + NC * NC)))
     wlap_kernel(const E *__restrict__ U, const E *__restrict__ in, E *__restrict__ out, Lat g,
                 typename Acc<E>::T centre) {
     using A = typename Acc<E>::T;
@@ -138,7 +139,8 @@ __global__ void __launch_bounds__(stencil_max_threads(MINB), (MINB > 1 ? 1 : 0))
 // STAGED: W~ through shared memory, one ring per block (wstage.cuh); else each
 // thread reads its own.
 template <int NC, int NS, int VR, typename E, int MINB, int LAYOUT, bool STAGED>
-__global__ void __launch_bounds__(stencil_max_threads(MINB), (MINB > 1 ? 1 : 0))
+__global__ void __launch_bounds__(stencil_max_threads(MINB),
+                                  (stencil_min_blocks<NC, NS, VR, MINB, typename Acc<E>::T>(NC >= 4, NC * NS * VR + NC * NC)))
     blap_kernel(const E *__restrict__ W, const E *__restrict__ in, E *__restrict__ out, Lat g,
                 typename Acc<E>::T centre) {
     using A = typename Acc<E>::T;
@@ -241,6 +243,7 @@ template <typename E, int LAYOUT>
 int launch_laplace_v(const dirac_op *op, const void *in, void *out, double m, cudaStream_t s) {
     int vr, minb, block;
     launch_variant(op, vr, minb, block);
+    vr = aligned_vr(vr, op->prec, in, out);
     using A = typename Acc<E>::T;
     const bool bril = uses_w(op->kind);
     const double centre = bril ? 0.5 * m * m + 240.0 / 128.0 : 4.0 + 0.5 * m * m;

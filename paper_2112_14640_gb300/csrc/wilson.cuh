@@ -150,9 +150,10 @@ __device__ __forceinline__ void wilson_dir(cx<A> (&acc)[NC][4][VR], const EL *__
     const long long fw = neighbour(g, n, c, MU, +1);
     const long long bw = neighbour(g, n, c, MU, -1);
     const long long cs = L::cs_stride(g), ls = L::template mat_stride<NC>(g);
-    if constexpr (NC <= kMaxNcSmall) {
+    if constexpr (NC <= kTunedNc) {
         // both links of the direction are requested before either hop, so
-        // their loads are in flight together
+        // their loads are in flight together (N_c = 4: the second link's
+        // registers cost more warps than that hides)
         cx<A> Lf[NC][NC], Lb[NC][NC];
         load_mat_s<NC, EL, A>(U + 2 * L::template mat<NC>(g, n, 4, MU), ls, Lf);
         load_mat_s<NC, EL, A>(U + 2 * L::template mat<NC>(g, bw, 4, MU), ls, Lb);
@@ -170,9 +171,11 @@ __device__ __forceinline__ void wilson_dir(cx<A> (&acc)[NC][4][VR], const EL *__
 }
 
 template <int NC, int VR, typename E, int MINB, int LAYOUT, typename EL, int CLOV>
-__global__ void __launch_bounds__(stencil_max_threads(MINB), (MINB > 1 ? 1 : 0)) wilson_kernel(const EL *__restrict__ U, const E *__restrict__ in,
-                                                     E *__restrict__ out, Lat g, typename Acc<E>::T diag,
-                                                     typename Acc<E>::T sgn, const EL *__restrict__ clov) {
+__global__ void __launch_bounds__(stencil_max_threads(MINB),
+                                  (stencil_min_blocks<NC, 4, VR, MINB, typename Acc<E>::T>(
+                                      NC == 2 || NC == 4, 2 * NC * VR + (NC <= kMaxNcSmall ? NC * NC : NC))))
+    wilson_kernel(const EL *__restrict__ U, const E *__restrict__ in, E *__restrict__ out, Lat g,
+                  typename Acc<E>::T diag, typename Acc<E>::T sgn, const EL *__restrict__ clov) {
     using A = typename Acc<E>::T;
     const int nchunk = g.nv / VR;
     const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -204,6 +207,7 @@ template <typename E, int LAYOUT, typename EL>
 int launch_wilson_v(const dirac_op *op, const void *in, void *out, double m0, int sgn, cudaStream_t s) {
     int vr, minb, block;
     launch_variant(op, vr, minb, block);
+    vr = aligned_vr(vr, op->prec, in, out);
     using A = typename Acc<E>::T;
     return dispatch_nc<big_nc_ok<E>()>(op->nc, [&](auto ncc) {
         constexpr int NC = decltype(ncc)::value;
