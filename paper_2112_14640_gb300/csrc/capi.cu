@@ -36,6 +36,7 @@ namespace dgb {
     } while (0)
 
 int op_apply(const dirac_op *op, const void *in, void *out, double m0, int sgn, cudaStream_t s) {
+    if (split_applies(op)) return launch_split(op, in, out, m0, sgn, s);
     switch (op->kind) {
     case DIRAC_WILSON: return launch_wilson(op, in, out, m0, sgn, s);
     case DIRAC_BRILLOUIN: return launch_brillouin(op, in, out, m0, sgn, s);
@@ -437,11 +438,15 @@ int dirac_op_autotune(dirac_op *op, double m0, void *stream, double *best_ms) {
         float ms;
     };
     std::vector<Cand> cands;
+    dirac_op untuned = *op;
+    untuned.vr = 0;
+    const bool split = split_applies(&untuned);   // one kernel without variants
+    if (split) cands.push_back(Cand{0, 0, 0, 1e30f});
     const int vrs[3] = {1, 2, 4}, minbs[5] = {1, 3, 4, 5, 6}, blocks[5] = {128, 256, 384, 512, 768};
     for (int vr : vrs)
         for (int mb : minbs)
             for (int bl : blocks)
-                if (variant_ok(op, vr, mb) && bl <= stencil_max_threads(mb))
+                if (!split && variant_ok(op, vr, mb) && bl <= stencil_max_threads(mb))
                     cands.push_back(Cand{vr, mb, bl, 1e30f});
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);

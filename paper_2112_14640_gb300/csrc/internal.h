@@ -270,6 +270,10 @@ int launch_brillouin(const dirac_op *op, const void *in, void *out, double m0, i
 // A = -1/2 Lap + m^2/2 for the Laplace kinds (laplace.cuh); m is the mass of A
 int launch_laplace(const dirac_op *op, const void *in, void *out, double m, cudaStream_t s);
 
+// FP64 applies on small lattices with the hops of a site spread over lanes (split.cu)
+bool split_applies(const dirac_op *op);
+int launch_split(const dirac_op *op, const void *in, void *out, double m0, int sgn, cudaStream_t s);
+
 // link preparation
 int launch_phase_links(dirac_op *op, const void *U, dirac_prec u_prec, cudaStream_t s);
 int launch_build_w(dirac_op *op, const void *U, dirac_prec u_prec, cudaStream_t s);
