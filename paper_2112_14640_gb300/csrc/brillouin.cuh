@@ -468,8 +468,8 @@ int launch_brillouin_v(const dirac_op *op, const void *in, void *out, double m0,
                     return launch_check("brillouin_kernel");
                 };
                 const size_t smem = NC <= kMaxNcSmall ? wst::smem_bytes<NC, EL>(block, nchunk) : 0;
-                if (NC > kMaxNcSmall || nchunk < wst::kMinChunks || smem > wst::kMaxSmem) {
-                    // few threads share a site's W~: compiled for two register classes only
+                if (NC > kMaxNcSmall || nchunk < wst::kMinChunks<EL> || smem > wst::kMaxSmem) {
+                    // W~ read by each thread: compiled for two register classes only
                     if constexpr (NC == 3 && VR == 1) {
                         if (minb > 1) return go(brillouin_kernel<NC, VR, E, 4, LAYOUT, EL, false>, block <= 512 ? block : 512, 0);
                     }

@@ -235,8 +235,12 @@ inline void launch_variant(const dirac_op *op, int &vr, int &minb, int &block) {
     block = kStencilBlock;
     // D_S reads 24 N_v bytes a site beside 72 of links per hop: the widest
     // group of one 32-byte access spreads a link over the most RHS (16^3x32,
-    // N_v = 12, FP32: 36 us, two RHS per thread 41 us)
-    if (op->kind == DIRAC_STAGGERED && op->prec == DIRAC_F32 && op->nc <= kMaxNcSmall && op->nv % 4 == 0) vr = 4;
+    // N_v = 12, FP32: 36 us, two RHS per thread 41 us; 16^4, N_v = 8: 12.4 and
+    // 14.3), while that leaves two warps per quarter-SM (D^dag D on 14x8x26x8,
+    // N_v = 4: 15.1 us, two RHS 12.6)
+    if (op->kind == DIRAC_STAGGERED && op->prec == DIRAC_F32 && op->nc <= kMaxNcSmall && op->nv % 4 == 0 &&
+        op->V * op->nv / 4 >= 2 * 608 * 32)
+        vr = 4;
     if (op->nc == 3) {
         if (op->kind == DIRAC_WILSON) minb = vr == 4 ? 3 : 4;
         else if (op->kind == DIRAC_STAGGERED) minb = vr == 4 ? 5 : 6;
@@ -249,6 +253,11 @@ inline void launch_variant(const dirac_op *op, int &vr, int &minb, int &block) {
         vr = op->nc >= 3 || vr == 1 ? 1 : 2;
         if (op->nc == 3) minb = 4;
     }
+    // bsuv with few threads per site: with the compiler's own choice of registers
+    // a block holds fewer warps than its ring allows (18x10x14x14, N_v = 3: 88 us,
+    // with a class 66; 13x9x5x4, N_v = 5: 32 and 19; but 22x13x25x4, N_v = 23: 171
+    // and 207)
+    if (op->kind == DIRAC_BSUV && op->prec == DIRAC_F32 && op->nc == 3 && op->nv / vr < 8) minb = 4;
 }
 
 // VR complex numbers of an element are one access of up to 32 bytes, which

@@ -281,8 +281,7 @@ int launch_laplace_v(const dirac_op *op, const void *in, void *out, double m, cu
                         });
                     });
                 const size_t smem = NC <= kMaxNcSmall ? wst::smem_bytes<NC, E>(block, nchunk) : 0;
-                if (NC > kMaxNcSmall || nchunk < wst::kMinChunks || smem > wst::kMaxSmem)
-                    // few threads share a site's W~
+                if (NC > kMaxNcSmall || nchunk < wst::kMinChunks<E> || smem > wst::kMaxSmem)
                     return on_spins([&](auto nsc) {
                         constexpr int NS = decltype(nsc)::value;
                         return run_w(blap_kernel<NC, NS, VR, E, 1, LAYOUT, false>,

@@ -38,12 +38,14 @@ template <int NC, typename EL>
 inline size_t smem_bytes(int T, int nchunk) {
     return (size_t)kRing * block_sites(T, nchunk) * Shape<NC, EL>::pitch;
 }
-// Staging pays where several threads share a site's matrices and a block's
-// ring leaves room for a few blocks per SM: at 16^3x32, FP32, N_v = 4 (four
-// threads per site) D_B takes 0.394 ms staged and 0.486 ms as two threads per
-// site reading their own; with fewer threads per site the ring of a block
-// grows past what leaves enough warps per SM.
-constexpr int kMinChunks = 4;
+// Staging pays wherever a block's ring leaves room for two blocks per SM, also
+// with few threads per site: FP32, N_c = 3, 18x10x14x14, read by each thread
+// and staged: D_B N_v = 3: 168 and 113 us, N_v = 2: 124 and 96, blap N_v = 3: 168
+// and 109, bsuv N_v = 3: 120 and 88; N_c = 2, N_v = 2, 31x14x15x18: 224 and 150.
+// (N_c = 3, N_v = 1 does not fit.)  FP64 is bound by its own pipe: there only
+// where four threads share a site, as the ring of fewer is too large at N_c = 3.
+template <typename EL>
+constexpr int kMinChunks = sizeof(EL) == 8 ? 4 : 1;
 constexpr size_t kMaxSmem = 100 * 1024;
 
 template <int BYTES>
