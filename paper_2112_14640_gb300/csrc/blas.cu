@@ -5,16 +5,23 @@
 // Reductions (norm^2, dot) carry at least FP64-like precision whatever the
 // storage precision (Sec. 3 accumulates sp norms in dp) and are
 // deterministic: a fixed grid of blocks, thread (r, v) of a block owns column
-// v, partial sums are combined in a fixed tree inside the block and then
-// summed in block order by a second one-block kernel.  FP64 vectors
-// accumulate in FP64.  FP32 and 16-bit vectors accumulate per thread in FP32
-// with error-free transformations (Dekker's product, Knuth's two-sum): every
-// product is split exactly into a rounded part and its error, the rounded
-// parts are summed with their rounding errors collected, and the pair
-// (sum, error) goes to the FP64 block reduction.  That keeps the thread
-// loops on the FP32 pipe: FP64 arithmetic on this GPU runs at a small
+// v, the threads' sums are combined in a fixed tree inside the block, and the
+// blocks' rows in a fixed order by a second kernel with a block per column (in
+// the CG passes by the last block to finish).  FP64 vectors accumulate in
+// FP64.  FP32 and 16-bit vectors accumulate per thread in FP32 with error-free
+// transformations (Dekker's product, Knuth's two-sum): every product is split
+// exactly into a rounded part and its error, and the rounded parts are summed
+// with their rounding errors collected in a pair (sum, error).  That keeps the
+// thread loops on the FP32 pipe: FP64 arithmetic on this GPU runs at a small
 // fraction of the FP32 rate and would limit the reductions far below HBM
 // bandwidth.
+//
+// Across threads the sums are added as FP64 would or better.  FP64 additions of
+// every thread's sum cost as much as a small reduction (8^4, N_v = 3: 2.3 us
+// more per CG pass), so while it stays in FP32's range a column is added up as
+// three floats (72 bits); a column that leaves it is added up once more, from
+// the threads' own sums, in FP64.  Only a single thread's share of the rows is
+// bound to the range of FP32.
 //
 // Every thread handles four rows per loop trip so that four independent
 // 16-byte loads per operand are in flight.
@@ -32,13 +39,13 @@ inline int blas_group(dirac_prec p, int nv) { return pick_vr(p, nv); }
 // Threads per block: a multiple of the number of column groups nv/G.
 inline int red_block(int ngroups) { return ngroups * (kRedThreads / ngroups); }
 
-// Per-thread accumulator of a real sum.  FP64 data: a plain double.  FP32
-// data: (s, c) with the exact value s + c of everything added so far up to
-// the errors of the error-free steps (Knuth's two-sum and Dekker's product via
-// FMA); the explicit __f*_rn intrinsics keep the compiler from contracting or
-// reassociating them.  Either is eight bytes, and two of them join without
-// leaving the FP32 pipe, so a block's and a launch's partial sums stay in this
-// form: FP64 additions of every thread's sum cost as much as a small reduction.
+// Accumulator of a real sum.  FP64 data: a plain double.  FP32 data: the
+// exact value s + c (+ e) of everything added so far up to the errors of the
+// error-free steps (Knuth's two-sum and Dekker's product via FMA); the explicit
+// __f*_rn intrinsics keep the compiler from contracting or reassociating them.
+// A thread's own sum is the pair (s, c); joining two accumulators also keeps
+// the rounding errors of c, in e, so that it adds nothing to the error of an
+// FP64 number.  Once s has left FP32's range it is infinite or NaN and stays so.
 template <typename A>
 struct RedAcc;
 template <>
@@ -47,92 +54,133 @@ struct RedAcc<double> {
     __device__ __forceinline__ void mac(double x, double y) { s = fma(x, y, s); }
     __device__ __forceinline__ void join(const RedAcc &o) { s += o.s; }
     __device__ __forceinline__ RedAcc down(int lanes) const { return RedAcc{__shfl_down_sync(~0u, s, lanes)}; }
+    __device__ __forceinline__ bool in_range() const { return true; }
     __device__ __forceinline__ double value() const { return s; }
 };
 template <>
-struct __align__(8) RedAcc<float> {
-    float s = 0.f, c = 0.f;
-    __device__ __forceinline__ void add(float p) {
-        const float t = __fadd_rn(s, p);
-        const float bp = __fsub_rn(t, s);
-        c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(p, bp)));
-        s = t;
+struct RedAcc<float> {
+    float s = 0.f, c = 0.f, e = 0.f;
+    // a + b = sum + err exactly
+    static __device__ __forceinline__ void two_sum(float a, float b, float &sum, float &err) {
+        const float t = __fadd_rn(a, b);
+        const float bp = __fsub_rn(t, a);
+        err = __fadd_rn(__fsub_rn(a, __fsub_rn(t, bp)), __fsub_rn(b, bp));
+        sum = t;
     }
     __device__ __forceinline__ void mac(float x, float y) {
         const float p = __fmul_rn(x, y);
-        add(p);
+        float err;
+        two_sum(s, p, s, err);
+        c = __fadd_rn(c, err);
         c = __fadd_rn(c, __fmaf_rn(x, y, -p));
     }
     __device__ __forceinline__ void join(const RedAcc &o) {
-        add(o.s);
-        c = __fadd_rn(c, o.c);
+        float e1, e2, e3;
+        two_sum(s, o.s, s, e1);
+        two_sum(c, o.c, c, e2);
+        two_sum(c, e1, c, e3);
+        e = __fadd_rn(__fadd_rn(e, o.e), __fadd_rn(e2, e3));
     }
     __device__ __forceinline__ RedAcc down(int lanes) const {
-        return RedAcc{__shfl_down_sync(~0u, s, lanes), __shfl_down_sync(~0u, c, lanes)};
+        return RedAcc{__shfl_down_sync(~0u, s, lanes), __shfl_down_sync(~0u, c, lanes), __shfl_down_sync(~0u, e, lanes)};
     }
-    __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+    __device__ __forceinline__ bool in_range() const { return fabsf(s) <= 3.4028234e38f; }
+    __device__ __forceinline__ double value() const { return (double)s + ((double)c + (double)e); }
+};
+
+// A block's sum of a column as it goes to the last block of a CG pass: an
+// accumulator, or an FP64 number where the accumulator has no range for it.
+template <typename A>
+struct RedRow;
+template <>
+struct RedRow<double> {
+    double v;
+    static __device__ __forceinline__ RedRow wide(double v) { return RedRow{v}; }
+    static __device__ __forceinline__ RedRow of(const RedAcc<double> &a) { return RedRow{a.s}; }
+    static __device__ __forceinline__ RedRow load(const RedRow *p) { return RedRow{__ldcg(&p->v)}; }
+    __device__ __forceinline__ bool is_wide() const { return false; }
+    __device__ __forceinline__ RedAcc<double> acc() const { return RedAcc<double>{v}; }
+    __device__ __forceinline__ double value() const { return v; }
+};
+template <>
+struct RedRow<float> {
+    float4 v;   // s, c, e, 0; or the two words of a double, unused, 1
+    static __device__ __forceinline__ RedRow wide(double d) {
+        return RedRow{make_float4(__int_as_float(__double2loint(d)), __int_as_float(__double2hiint(d)), 0.f, 1.f)};
+    }
+    static __device__ __forceinline__ RedRow of(const RedAcc<float> &a) { return RedRow{make_float4(a.s, a.c, a.e, 0.f)}; }
+    static __device__ __forceinline__ RedRow load(const RedRow *p) { return RedRow{__ldcg(&p->v)}; }
+    __device__ __forceinline__ bool is_wide() const { return v.w != 0.f; }
+    __device__ __forceinline__ RedAcc<float> acc() const { return RedAcc<float>{v.x, v.y, v.z}; }
+    __device__ __forceinline__ double value() const {
+        return is_wide() ? __hiloint2double(__float_as_int(v.y), __float_as_int(v.x)) : acc().value();
+    }
 };
 
 // Rows of a column in shared memory: [column][row], an odd pitch.
 __host__ __device__ constexpr int red_pitch(int rows) { return rows | 1; }
 
-// Join the `rows` sums of every column, one warp per column at a time: lanes
-// take rows lane, lane + 32, ..., then a fixed tree; put(column, sum) runs in
-// lane 0.  Whole warps only (blocks need not be a multiple of 32 threads).
+// Sum of get(0 .. rows - 1) in FP64 by one warp, in lane 0: lanes take rows
+// lane, lane + 32, ..., then a fixed tree.
+template <typename GET>
+__device__ __forceinline__ double warp_sum(int rows, GET get) {
+    double acc = 0.0;
+    for (int r = threadIdx.x & 31; r < rows; r += 32) acc += get(r);
+    for (int off = 16; off > 0; off /= 2) acc += __shfl_down_sync(~0u, acc, off);
+    return acc;
+}
+
+// Join the `rows` sums of every column, one warp per column at a time, in the
+// order of warp_sum; put(column, row) runs in lane 0.  Whole warps only
+// (blocks need not be a multiple of 32 threads).
 template <typename A, typename PUT>
 __device__ __forceinline__ void join_columns(const RedAcc<A> *sh, int cols, int rows, PUT put) {
     const int nwarps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp >= nwarps) return;
     for (int c = warp; c < cols; c += nwarps) {
+        const RedAcc<A> *col = sh + c * red_pitch(rows);
         RedAcc<A> acc;
-        for (int r = lane; r < rows; r += 32) acc.join(sh[c * red_pitch(rows) + r]);
+        for (int r = lane; r < rows; r += 32) acc.join(col[r]);
         for (int off = 16; off > 0; off /= 2) acc.join(acc.down(off));
-        if (lane == 0) put(c, acc);
+        RedRow<A> row = RedRow<A>::of(acc);
+        if (__any_sync(~0u, lane == 0 && !acc.in_range()))
+            row = RedRow<A>::wide(warp_sum(rows, [&](int r) { return col[r].value(); }));
+        if (lane == 0) put(c, row);
     }
 }
 
-// The sums vals[G][NOUT] of the R row-threads of a block, joined per column
-// and stored as the block's row of partial sums: partial_block[v NOUT + q].
-template <int G, int NOUT, typename A>
-__device__ __forceinline__ void block_reduce_store(const RedAcc<A> (&vals)[G][NOUT], RedAcc<A> *sh, int r, int vg, int R,
-                                                   int ng, RedAcc<A> *partial_block) {
+// The sums vals[G][NOUT] of the R row-threads of a block, joined per column;
+// put(v NOUT + q, row) for each.
+template <int G, int NOUT, typename A, typename PUT>
+__device__ __forceinline__ void block_reduce(const RedAcc<A> (&vals)[G][NOUT], RedAcc<A> *sh, int r, int vg, int R,
+                                             int ng, PUT put) {
     if (r < R)
 #pragma unroll
         for (int i = 0; i < G; ++i)
 #pragma unroll
             for (int q = 0; q < NOUT; ++q) sh[((vg * G + i) * NOUT + q) * red_pitch(R) + r] = vals[i][q];
     __syncthreads();
-    join_columns(sh, ng * G * NOUT, R, [&](int c, const RedAcc<A> &v) { partial_block[c] = v; });
+    join_columns(sh, ng * G * NOUT, R, put);
 }
 
-// Second pass of a reduction: partial[b][col] (col = v*NOUT + q, cols =
-// nv*NOUT) -> out[col].  One block of kFinThreads threads: T = kFinThreads /
-// cols threads per column each join the blocks t, t+T, ... in order, then the
-// T sums, so the result does not depend on timing.
+// Second pass of a reduction: partial[b][col] (col = v*NOUT + q) -> out[col],
+// one block per column, so that the columns' FP64 additions run side by side.
+// The order is fixed by the number of blocks.
 constexpr int kFinThreads = 256;
-template <int NOUT, typename A>
-__global__ void __launch_bounds__(kFinThreads) finalize_kernel(const RedAcc<A> *__restrict__ partial, int nblocks,
-                                                               int nv, double *__restrict__ out) {
-    __shared__ double raw[2 * kFinThreads];   // cols rows of T | 1
-    RedAcc<A> *sh = reinterpret_cast<RedAcc<A> *>(raw);
-    const int cols = nv * NOUT;
-    const int T = kFinThreads / cols;
-    const int t = threadIdx.x / cols, c = threadIdx.x % cols;
-    RedAcc<A> acc;
-    if (t < T) {
-        constexpr int U = 8;   // rows in flight per thread
-        for (int b0 = t; b0 < nblocks; b0 += U * T) {
-            RedAcc<A> in[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (b0 + u * T < nblocks) in[u] = partial[(long long)(b0 + u * T) * cols + c];
-#pragma unroll
-            for (int u = 0; u < U; ++u) acc.join(in[u]);   // zero past the last row
-        }
-        sh[c * red_pitch(T) + t] = acc;
-    }
+__global__ void __launch_bounds__(kFinThreads) finalize_kernel(const double *__restrict__ partial, int nblocks,
+                                                               double *__restrict__ out) {
+    __shared__ double sh[kFinThreads / 32];
+    const int cols = gridDim.x, c = blockIdx.x, warp = threadIdx.x / 32;
+    // warp w adds up the rows 32 w .. 32 w + 31 of every 256
+    double acc = 0.0;
+    for (int b = threadIdx.x; b < nblocks; b += kFinThreads) acc += partial[(long long)b * cols + c];
+    const double sum = warp_sum(32, [&](int) { return acc; });
+    if (threadIdx.x % 32 == 0) sh[warp] = sum;
     __syncthreads();
-    join_columns(sh, cols, T, [&](int col, const RedAcc<A> &v) { out[col] = v.value(); });
+    if (warp == 0) {
+        const double all = warp_sum(kFinThreads / 32, [&](int w) { return sh[w]; });
+        if (threadIdx.x == 0) out[c] = all;
+    }
 }
 
 // thread (r, vg) of a block walks the rows r0 = block*R + r, stride grid*R and
@@ -156,8 +204,7 @@ struct RowMap {
 
 template <typename E, int G>
 __global__ void norm2_kernel(const E *__restrict__ x, long long rows, int nv,
-                             RedAcc<typename Acc<E>::T> *__restrict__ partial,
-                             RowMap rm = RowMap{}) {
+                             double *__restrict__ partial, RowMap rm = RowMap{}) {
     extern __shared__ __align__(8) unsigned char red_smem[];
     using A = typename Acc<E>::T;
     RedAcc<A> *sh = reinterpret_cast<RedAcc<A> *>(red_smem);
@@ -185,12 +232,13 @@ __global__ void norm2_kernel(const E *__restrict__ x, long long rows, int nv,
             add(a[0]);
         }
     }
-    block_reduce_store<G, 1, A>(acc, sh, r, vg, R, ng, partial + (long long)blockIdx.x * nv);
+    block_reduce(acc, sh, r, vg, R, ng,
+                 [&](int c, const RedRow<A> &v) { partial[(long long)blockIdx.x * nv + c] = v.value(); });
 }
 
 template <typename E, int G>
 __global__ void dot_kernel(const E *__restrict__ x, const E *__restrict__ y, long long rows, int nv,
-                           RedAcc<typename Acc<E>::T> *__restrict__ partial, RowMap rm = RowMap{}) {
+                           double *__restrict__ partial, RowMap rm = RowMap{}) {
     extern __shared__ __align__(8) unsigned char red_smem[];
     using A = typename Acc<E>::T;
     RedAcc<A> *sh = reinterpret_cast<RedAcc<A> *>(red_smem);
@@ -226,7 +274,8 @@ __global__ void dot_kernel(const E *__restrict__ x, const E *__restrict__ y, lon
             add(a[0], b[0]);
         }
     }
-    block_reduce_store<G, 2, A>(acc, sh, r, vg, R, ng, partial + 2LL * blockIdx.x * nv);
+    block_reduce(acc, sh, r, vg, R, ng,
+                 [&](int c, const RedRow<A> &v) { partial[2LL * blockIdx.x * nv + c] = v.value(); });
 }
 
 template <typename A>
@@ -240,7 +289,7 @@ __device__ __forceinline__ cx<A> coef(const double *c, double scale, int v) {
 template <typename E, int G>
 __global__ void axpby_kernel(E *z, const E *x, const E *y, const double *__restrict__ ac, double as,
                              const double *__restrict__ bc, double bs, long long rows, int nv,
-                             RedAcc<typename Acc<E>::T> *partial) {
+                             double *partial) {
     extern __shared__ __align__(8) unsigned char red_smem[];
     using A = typename Acc<E>::T;
     RedAcc<A> *sh = reinterpret_cast<RedAcc<A> *>(red_smem);
@@ -295,9 +344,9 @@ __global__ void axpby_kernel(E *z, const E *x, const E *y, const double *__restr
             finish(e, tx[0], ty[0]);
         }
     }
-    if (partial) {
-        block_reduce_store<G, 1, A>(acc, sh, r, vg, R, ng, partial + (long long)blockIdx.x * nv);
-    }
+    if (partial)
+        block_reduce(acc, sh, r, vg, R, ng,
+                     [&](int c, const RedRow<A> &v) { partial[(long long)blockIdx.x * nv + c] = v.value(); });
 }
 
 // ------------------------------------------------------------ CG kernels
@@ -311,18 +360,11 @@ __global__ void axpby_kernel(E *z, const E *x, const E *y, const double *__restr
 // 6 TB/s), bound by the chain load - reduce - last block on small ones (8^4,
 // N_v = 3: about 5, 6 and 3 us).
 
-// Join the blocks' partial rows (nv sums each) in the last block to arrive;
-// the N_v values there, null in every other block.  Fixed order, so
-// reproducible.  This block's row was written before the call.
-__device__ __forceinline__ RedAcc<double> load_cg(const RedAcc<double> *p) {
-    return RedAcc<double>{__ldcg(reinterpret_cast<const double *>(p))};
-}
-__device__ __forceinline__ RedAcc<float> load_cg(const RedAcc<float> *p) {
-    const float2 f = __ldcg(reinterpret_cast<const float2 *>(p));
-    return RedAcc<float>{f.x, f.y};
-}
+// Join the blocks' rows (nv sums each) in the last block to arrive; the N_v
+// values there, null in every other block.  Fixed order, so reproducible.
+// This block's row was written before the call.
 template <typename A>
-__device__ __forceinline__ const double *last_block_sum(const RedAcc<A> *partial, unsigned *counter, int nv,
+__device__ __forceinline__ const double *last_block_sum(const RedRow<A> *partial, unsigned *counter, int nv,
                                                         RedAcc<A> *sh) {
     __shared__ bool last;
     __shared__ double sums[64];
@@ -333,21 +375,36 @@ __device__ __forceinline__ const double *last_block_sum(const RedAcc<A> *partial
     if (!last) return nullptr;
     __threadfence();
     const int T = blockDim.x / nv, t = threadIdx.x / nv, c = threadIdx.x - t * nv;
+    bool wide = false;
     if (t < T) {
         RedAcc<A> acc;
         constexpr int U = 8;   // rows in flight per thread
         for (int b0 = t; b0 < (int)gridDim.x; b0 += U * T) {
-            RedAcc<A> in[U];
+            RedRow<A> in[U];
 #pragma unroll
             for (int u = 0; u < U; ++u)
-                if (b0 + u * T < (int)gridDim.x) in[u] = load_cg(partial + (long long)(b0 + u * T) * nv + c);
+                in[u] = b0 + u * T < (int)gridDim.x ? RedRow<A>::load(partial + (long long)(b0 + u * T) * nv + c)
+                                                    : RedRow<A>::of(RedAcc<A>{});   // zero past the last row
 #pragma unroll
-            for (int u = 0; u < U; ++u) acc.join(in[u]);   // zero past the last row
+            for (int u = 0; u < U; ++u) {
+                wide |= in[u].is_wide();
+                acc.join(in[u].acc());
+            }
         }
+        wide |= !acc.in_range();
         sh[c * red_pitch(T) + t] = acc;
     }
-    __syncthreads();
-    join_columns(sh, nv, T, [&](int col, const RedAcc<A> &v) { sums[col] = v.value(); });
+    if (__syncthreads_or(wide)) {
+        const int nwarps = blockDim.x >> 5, warp = threadIdx.x >> 5;
+        for (int v = warp; v < nv && warp < nwarps; v += nwarps) {
+            const double sum = warp_sum(gridDim.x, [&](int b) {
+                return RedRow<A>::load(partial + (long long)b * nv + v).value();
+            });
+            if ((threadIdx.x & 31) == 0) sums[v] = sum;
+        }
+    } else {
+        join_columns(sh, nv, T, [&](int col, const RedRow<A> &v) { sums[col] = v.value(); });
+    }
     __syncthreads();
     return sums;
 }
@@ -384,8 +441,9 @@ __global__ void cg_dot_kernel(const E *__restrict__ x, const E *__restrict__ y, 
             for (int u = 0; u < 4; ++u)
                 if (row + u * stride < rows) add(a[u], b[u]);
         }
-    RedAcc<A> *partial = reinterpret_cast<RedAcc<A> *>(k.partial);
-    block_reduce_store<G, 1, A>(acc, sh, r, vg, R, ng, partial + (long long)blockIdx.x * nv);
+    RedRow<A> *partial = reinterpret_cast<RedRow<A> *>(k.partial);
+    block_reduce(acc, sh, r, vg, R, ng,
+                 [&](int c, const RedRow<A> &v) { partial[(long long)blockIdx.x * nv + c] = v; });
     const double *sums = last_block_sum(partial, k.counter, nv, sh);
     if (!sums) return;
     const int v = threadIdx.x;
@@ -436,8 +494,9 @@ __global__ void cg_residual_kernel(E *rv, const E *__restrict__ q, long long row
             for (int u = 0; u < 4; ++u)
                 if (row + u * stride < rows) finish(2 * ((row + u * stride) * nv + vg * G), tr[u], tq[u]);
         }
-    RedAcc<A> *partial = reinterpret_cast<RedAcc<A> *>(k.partial);
-    block_reduce_store<G, 1, A>(acc, sh, r, vg, R, ng, partial + (long long)blockIdx.x * nv);
+    RedRow<A> *partial = reinterpret_cast<RedRow<A> *>(k.partial);
+    block_reduce(acc, sh, r, vg, R, ng,
+                 [&](int c, const RedRow<A> &v) { partial[(long long)blockIdx.x * nv + c] = v; });
     const double *sums = last_block_sum(partial, k.counter, nv, sh);
     if (!sums) return;
     const int v = threadIdx.x;
@@ -545,7 +604,7 @@ static RedLaunch red_launch(dirac_prec p, int nv, int nout) {
     const int ng = nv / L.G;
     L.tb = red_block(ng);
     // one extra row of slots absorbs the threads beyond R (tb is a multiple of ng)
-    L.sh = (size_t)(L.tb + ng) * L.G * nout * sizeof(double);
+    L.sh = (size_t)(L.tb + ng) * L.G * nout * (p == DIRAC_F64 ? sizeof(RedAcc<double>) : sizeof(RedAcc<float>));
     return L;
 }
 
@@ -636,21 +695,14 @@ int blas_fill_hash(const dirac_op *op, dirac_prec p, void *v, unsigned seed, cud
 
 static inline int red_grid(const dirac_op *op) { return op->red_blocks; }
 
-// the reduction buffer as partial sums of E's accumulators (eight bytes each)
-template <typename E>
-static RedAcc<typename Acc<E>::T> *partials(double *buf) {
-    return reinterpret_cast<RedAcc<typename Acc<E>::T> *>(buf);
-}
-
 template <typename E>
 static int launch_norm2(const E *v, long long rows, int nv, dirac_prec p, double *buf, int blocks, double *out,
                         cudaStream_t s) {
-    auto *partial = partials<E>(buf);
     const RedLaunch L = red_launch(p, nv, 1);
     return dispatch_group(L.G, [&](auto gc) {
         constexpr int G = decltype(gc)::value;
-        norm2_kernel<E, G><<<blocks, L.tb, L.sh, s>>>(v, rows, nv, partial);
-        finalize_kernel<1><<<1, kFinThreads, 0, s>>>(partial, blocks, nv, out);
+        norm2_kernel<E, G><<<blocks, L.tb, L.sh, s>>>(v, rows, nv, buf);
+        finalize_kernel<<<nv, kFinThreads, 0, s>>>(buf, blocks, out);
         return launch_check("norm2_kernel");
     });
 }
@@ -669,8 +721,8 @@ int blas_dot(const dirac_op *op, dirac_prec p, const void *u, const void *v, dou
         return dispatch_group(L.G, [&](auto gc) {
             constexpr int G = decltype(gc)::value;
             dot_kernel<E, G><<<red_grid(op), L.tb, L.sh, s>>>((const E *)u, (const E *)v, op->rows, op->nv,
-                                                              partials<E>(op->red_partial));
-            finalize_kernel<2><<<1, kFinThreads, 0, s>>>(partials<E>(op->red_partial), red_grid(op), op->nv, out);
+                                                              op->red_partial);
+            finalize_kernel<<<2 * op->nv, kFinThreads, 0, s>>>(op->red_partial, red_grid(op), out);
             return launch_check("dot_kernel");
         });
     });
@@ -702,8 +754,8 @@ int blas_norm2_range(const dirac_op *op, dirac_prec p, const void *v, long long 
         return dispatch_group(L.G, [&](auto gc) {
             constexpr int G = decltype(gc)::value;
             norm2_kernel<E, G><<<red_grid(op), L.tb, L.sh, s>>>((const E *)v + 2 * first * op->nv, rows, op->nv,
-                                                                partials<E>(op->red_partial), rm);
-            finalize_kernel<1><<<1, kFinThreads, 0, s>>>(partials<E>(op->red_partial), red_grid(op), op->nv, out);
+                                                                op->red_partial, rm);
+            finalize_kernel<<<op->nv, kFinThreads, 0, s>>>(op->red_partial, red_grid(op), out);
             return launch_check("norm2_kernel");
         });
     });
@@ -721,8 +773,8 @@ int blas_dot_range(const dirac_op *op, dirac_prec p, const void *u, const void *
             constexpr int G = decltype(gc)::value;
             dot_kernel<E, G><<<red_grid(op), L.tb, L.sh, s>>>((const E *)u + 2 * first * op->nv,
                                                               (const E *)v + 2 * first * op->nv, rows, op->nv,
-                                                              partials<E>(op->red_partial), rm);
-            finalize_kernel<2><<<1, kFinThreads, 0, s>>>(partials<E>(op->red_partial), red_grid(op), op->nv, out);
+                                                              op->red_partial, rm);
+            finalize_kernel<<<2 * op->nv, kFinThreads, 0, s>>>(op->red_partial, red_grid(op), out);
             return launch_check("dot_kernel");
         });
     });
@@ -737,8 +789,8 @@ int blas_axpby(const dirac_op *op, dirac_prec p, void *z, const void *x, const d
             constexpr int G = decltype(gc)::value;
             axpby_kernel<E, G><<<red_grid(op), L.tb, L.sh, s>>>((E *)z, (const E *)x, (const E *)y, a, as, b, bs,
                                                                 op->rows, op->nv,
-                                                                norm_out ? partials<E>(op->red_partial) : nullptr);
-            if (norm_out) finalize_kernel<1><<<1, kFinThreads, 0, s>>>(partials<E>(op->red_partial), red_grid(op), op->nv, norm_out);
+                                                                norm_out ? op->red_partial : nullptr);
+            if (norm_out) finalize_kernel<<<op->nv, kFinThreads, 0, s>>>(op->red_partial, red_grid(op), norm_out);
             return launch_check("axpby_kernel");
         });
     });

@@ -330,7 +330,7 @@ struct CgScalars {
     // of x and p is due (alpha and beta of the last iteration not yet used)
     int *ctl;
     double *hist;         // per iteration: <p, A p>, old |r|^2, new |r|^2 (3 nv)
-    double *partial;      // one row of nv doubles per block
+    double *partial;      // per block a row of nv sums (16 bytes each, 16-byte aligned)
     unsigned *counter;    // zero between launches
 };
 // pq = Re <p, q> and alpha = rr / pq

@@ -46,7 +46,8 @@ struct Ws {
 static int get_ws(const dirac_op *op, Ws &w) {
     dirac_op *self = (dirac_op *)op;
     constexpr int kArrays = 20, kRun = 2 + kCgHistory * 3 * kNS;
-    const size_t scal = (kArrays * kNS * 2 + kRun + 1 + (size_t)kCgBlocks * kNS) * sizeof(double);
+    // kRun is even, so with two for the counter `partial` starts on a multiple of 16 bytes
+    const size_t scal = (kArrays * kNS * 2 + kRun + 2 + (size_t)kCgBlocks * kNS * 2) * sizeof(double);
     const size_t need = kWsVecs * op->vec_bytes + scal;
     if (!self->solver_ws) {
         if (cudaMalloc(&self->solver_ws, need) != cudaSuccess) {
@@ -71,7 +72,7 @@ static int get_ws(const dirac_op *op, Ws &w) {
     for (size_t i = 0; i < sizeof(arr) / sizeof(arr[0]); ++i) *arr[i] = d + i * kNS * 2;
     w.run = d + kArrays * kNS * 2;
     w.counter = (unsigned *)(w.run + kRun);
-    w.partial = w.run + kRun + 1;
+    w.partial = w.run + kRun + 2;
     return DIRAC_OK;
 }
 
