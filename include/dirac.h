@@ -426,7 +426,9 @@ int dirac_solve(const dirac_op *op, const void *b, void *x, double m0,
  * nodes are unavailable).  stats (host array of nsolves, may be NULL) receive per-solve
  * iterations (segment granularity), final residuals and the device-timed
  * seconds from the batch start to that solve's completion.  Blocks until done.
- * Returns 0 when all converged, DIRAC_NOT_CONVERGED otherwise. */
+ * Returns 0 when all converged, DIRAC_NOT_CONVERGED otherwise.  A solve with a
+ * NaN or an infinity in a norm ends there, DIRAC_NONFINITE in its stats; the
+ * others go on. */
 int dirac_solve_batched(int nsolves, dirac_op *const *ops, const void *const *b, void *const *x,
                         const double *m0, const dirac_solve_params *params, dirac_solve_stats *stats,
                         void *stream);

@@ -36,30 +36,34 @@ __global__ void stamp_kernel(unsigned long long *t) {
 }
 
 // After a recompute: freeze the RHS whose true residual passes; when all have
-// passed, mark the solve done and stamp the time (first time only).
+// passed, mark the solve done and stamp the time (first time only).  A NaN or an
+// infinity in a norm ends the solve as well, as nonfinite.
 struct BatchState {
     int done;
+    int nonfinite;
     int iters;
     unsigned long long stamp;
 };
 
 __global__ void batch_check_kernel(int nv, const double *rr_true, const double *nb, double tol2, double *act,
                                    BatchState *st, int K, cudaGraphConditionalHandle cond, int set_cond) {
-    __shared__ int any;
+    __shared__ int any, bad;
     const int v = threadIdx.x;
-    if (v == 0) any = 0;
+    if (v == 0) any = bad = 0;
     __syncthreads();
     const int done = st->done;
     if (v < nv && !done) {
         const bool pass = !(rr_true[v] >= tol2 * nb[v]);
         act[v] = pass ? 0.0 : 1.0;
         if (!pass) atomicOr(&any, 1);
+        if (!isfinite(rr_true[v]) || !isfinite(nb[v])) atomicOr(&bad, 1);
     }
     __syncthreads();
     if (v == 0 && !done) {
         st->iters += K;
-        if (!any) {
+        if (bad || !any) {
             st->done = 1;
+            st->nonfinite = bad;
             st->stamp = globaltimer();
         }
     }
@@ -347,7 +351,7 @@ extern "C" int dirac_solve_batched(int nsolves, dirac_op *const *ops, const void
             TRYB(cuda_check(cudaMemcpy(nb, scal[i].nb, nv * sizeof(double), cudaMemcpyDeviceToHost), "D2H"));
             st.iters = hstate[i].iters;
             st.recomputes = hstate[i].iters / K;
-            st.status = hstate[i].done ? DIRAC_OK : DIRAC_NOT_CONVERGED;
+            st.status = hstate[i].nonfinite ? DIRAC_NONFINITE : hstate[i].done ? DIRAC_OK : DIRAC_NOT_CONVERGED;
             for (int v = 0; v < nv; ++v) {
                 st.relres[v] = nb[v] > 0 ? sqrt(rr[v] / nb[v]) : 0.0;
                 st.status_per_rhs[v] = (nb[v] == 0.0 || rr[v] < tol2 * nb[v]) ? DIRAC_OK : DIRAC_NOT_CONVERGED;
@@ -359,7 +363,7 @@ extern "C" int dirac_solve_batched(int nsolves, dirac_op *const *ops, const void
     rc = DIRAC_OK;
     {
         bool all = true;
-        for (int i = 0; i < nsolves; ++i) all &= hstate[i].done != 0;
+        for (int i = 0; i < nsolves; ++i) all &= hstate[i].done && !hstate[i].nonfinite;
         if (!all) rc = DIRAC_NOT_CONVERGED;
     }
 fail:

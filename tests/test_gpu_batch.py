@@ -61,3 +61,25 @@ def test_batched_solve_already_converged_and_hpd():
     assert stats[0]["host_launches"] == 1
     assert stats[1]["iters"] > 0
     assert torch.allclose(xs[1], x0, rtol=0, atol=1e-8 * x0.abs().max().item())
+
+
+@pytest.mark.parametrize("value", [float("nan"), 1e30])   # 1e30: |b|^2 is past FP32's range in one thread
+def test_a_nonfinite_solve_is_reported_and_the_others_finish(value):
+    m0 = 0.3
+    ops, bs, refs, bn = [], [], [], []
+    for i, (dims, nv) in enumerate([((4, 4, 4, 4), 3), ((4, 4, 2, 4), 2), ((4, 2, 4, 6), 5)]):
+        U = I.gauge_field(dims, 3, 0.4, 500 + i)
+        ops.append(D.DiracOp(D.WILSON, torch.from_numpy(U).cuda(), nv, (1, 1, 1, -1), D.F32, layout=i % 2))
+        refs.append(O.Operator(D.WILSON, U, (1, 1, 1, -1)))
+        bn.append(I.source(dims, 3, nv, 510 + i))
+        bs.append(to_device(ops[-1], bn[-1]))
+    bs[1].view(-1)[7] = value
+    xs, stats, rc = D.solve_batched(ops, bs, m0s=[m0] * 3, tol=1e-5, maxit=2000)
+    assert rc == 1 and [s["status"] for s in stats] == [0, 4, 0], (rc, stats)
+    assert stats[1]["status_per_rhs"].count(0) < 2
+    for i in (0, 2):
+        bN = refs[i].apply_dagger(bn[i], m0)
+        res = np.sqrt(O.norm2(bN - refs[i].apply_normal(to_numpy(ops[i], xs[i]), m0)) / O.norm2(bN))
+        assert np.all(res < 5e-5), (i, res)
+    for op in ops:
+        op.close()
