@@ -53,7 +53,7 @@ __global__ void batch_check_kernel(int nv, const double *rr_true, const double *
     __syncthreads();
     const int done = st->done;
     if (v < nv && !done) {
-        const bool pass = !(rr_true[v] >= tol2 * nb[v]);
+        const bool pass = nb[v] == 0.0 || rr_true[v] < tol2 * nb[v];   // b = 0: x stays, as in dirac_solve
         act[v] = pass ? 0.0 : 1.0;
         if (!pass) atomicOr(&any, 1);
         if (!isfinite(rr_true[v]) || !isfinite(nb[v])) atomicOr(&bad, 1);

@@ -83,3 +83,18 @@ def test_a_nonfinite_solve_is_reported_and_the_others_finish(value):
         assert np.all(res < 5e-5), (i, res)
     for op in ops:
         op.close()
+
+
+def test_a_zero_right_hand_side_has_converged():
+    dims, nv, m0 = (4, 4, 2, 4), 3, 0.3
+    U = I.gauge_field(dims, 3, 0.4, 520)
+    op = D.DiracOp(D.WILSON, torch.from_numpy(U).cuda(), nv, (1, 1, 1, -1), D.F64)
+    b = to_device(op, I.source(dims, 3, nv, 521))
+    b[..., 1] = 0
+    (x,), (st,), rc = D.solve_batched([op], [b], m0s=[m0], tol=1e-10, maxit=2000)
+    assert rc == 0 and st["status"] == 0 and st["status_per_rhs"] == [0, 0, 0], (rc, st)
+    assert torch.count_nonzero(x[..., 1]) == 0
+    xr, sr = op.solve(b, m0=m0, tol=1e-10, maxit=2000)
+    assert sr["status"] == 0 and sr["status_per_rhs"] == [0, 0, 0]
+    assert float((x - xr).abs().max()) <= 1e-8 * float(xr.abs().max())
+    op.close()
