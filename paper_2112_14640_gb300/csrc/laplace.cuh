@@ -48,42 +48,67 @@ __host__ __device__ constexpr OffsetTable make_offset_table() {
 static __constant__ bril::OffsetTable kLapOffsets = bril::make_offset_table();
 
 // Whether a hop multiplies its weight into the N_c x N_c matrix (N_c^2 complex
-// scalings) or into the NS VR N_c vector components it reads.
+// scalings) and its products into the running sum, or sums its own N_c
+// products first and adds that sum with the weight (one real multiply-add per
+// complex component).  Without many components per matrix the second costs no
+// more and its sums are short, so its error is the smaller.
 template <int NC, int NS, int VR>
 constexpr bool fold_weight() { return NS * VR > NC; }
 
+// The running sum of a component: of products P where they go into it
+// directly, a plain number where a hop's own sum is added.
+template <typename P, int NC, int NS, int VR, typename A>
+using LapAcc = std::conditional_t<fold_weight<NC, NS, VR>(), typename P::Acc, typename Prod<A, false>::Acc>;
+
 // acc[c][s] += f L psi(m) (or f L^dag psi(m)) for every spin component s
 template <typename P, int NC, int NS, int VR, bool DAG, typename E, typename A>
-__device__ __forceinline__ void lap_hop(typename P::Acc (&acc)[NC][NS][VR], const cx<A> (&L)[NC][NC],
+__device__ __forceinline__ void lap_hop(LapAcc<P, NC, NS, VR, A> (&acc)[NC][NS][VR], const cx<A> (&L)[NC][NC],
                                         const E *__restrict__ psi, long long cs_stride, A f) {
-    constexpr bool FOLD = fold_weight<NC, NS, VR>();
-    // one colour component of the neighbour at a time: column k of the matrix
-    // and NS VR vector components in registers
+    if constexpr (fold_weight<NC, NS, VR>()) {
+        // one colour component of the neighbour at a time: column k of the matrix
+        // and NS VR vector components in registers
 #pragma unroll
-    for (int k = 0; k < NC; ++k) {
-        typename P::Mul w[NC];
+        for (int k = 0; k < NC; ++k) {
+            typename P::Mul w[NC];
 #pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            const cx<A> u = DAG ? conj(L[k][c]) : L[c][k];
-            w[c] = P::mul(FOLD ? f * u : u);
+            for (int c = 0; c < NC; ++c) w[c] = P::mul(f * (DAG ? conj(L[k][c]) : L[c][k]));
+#pragma unroll
+            for (int s = 0; s < NS; ++s) {
+                cx<A> p[VR];
+                load_cx<E, VR, A>(psi + 2 * (k * NS + s) * cs_stride, p);
+#pragma unroll
+                for (int v = 0; v < VR; ++v) {
+                    const typename P::Vec pv = P::vec(p[v]);
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) acc[c][s][v].mac(w[c], pv);
+                }
+            }
         }
+    } else {
 #pragma unroll
         for (int s = 0; s < NS; ++s) {
-            cx<A> p[VR];
-            load_cx<E, VR, A>(psi + 2 * (k * NS + s) * cs_stride, p);
+            cx<A> p[NC][VR];
 #pragma unroll
-            for (int v = 0; v < VR; ++v) {
-                const typename P::Vec pv = FOLD ? P::vec(p[v]) : P::scale(f, P::vec(p[v]));
+            for (int k = 0; k < NC; ++k) load_cx<E, VR, A>(psi + 2 * (k * NS + s) * cs_stride, p[k]);
 #pragma unroll
-                for (int c = 0; c < NC; ++c) acc[c][s][v].mac(w[c], pv);
+            for (int c = 0; c < NC; ++c) {
+                typename P::Acc t[VR];
+#pragma unroll
+                for (int k = 0; k < NC; ++k) {
+                    const typename P::Mul w = P::mul(DAG ? conj(L[k][c]) : L[c][k]);
+#pragma unroll
+                    for (int v = 0; v < VR; ++v) t[v].mac(w, P::vec(p[k][v]));
+                }
+#pragma unroll
+                for (int v = 0; v < VR; ++v) rmac(acc[c][s][v].s, f, t[v].value());
             }
         }
     }
 }
 
 template <typename P, int NC, int NS, int VR, int LAYOUT, typename E, typename A>
-__device__ __forceinline__ void lap_write(const E *__restrict__ in, E *__restrict__ out, const Lat &g,
-                                          long long n, int j, A centre, const typename P::Acc (&acc)[NC][NS][VR]) {
+__device__ __forceinline__ void lap_write(const E *__restrict__ in, E *__restrict__ out, const Lat &g, long long n,
+                                          int j, A centre, const LapAcc<P, NC, NS, VR, A> (&acc)[NC][NS][VR]) {
     using L = Layout<LAYOUT>;
     const long long cs = L::cs_stride(g);
     const long long base = 2 * (L::vec(g, n, NC * NS, 0) + (long long)j * VR);
@@ -120,7 +145,7 @@ __global__ void __launch_bounds__(stencil_max_threads(MINB),
 
     using P = Prod<A, false>;   // packed products measured slower here (0.121 vs 0.115 ms): the second
                                 // accumulator costs warps, and the loads bound this kernel
-    typename P::Acc acc[NC][NS][VR];
+    LapAcc<P, NC, NS, VR, A> acc[NC][NS][VR];
     const A mhalf = (A)-0.5;
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
@@ -175,7 +200,7 @@ __global__ void __launch_bounds__(stencil_max_threads(MINB),
         }
     }
     using P = StencilProd<NC, NS, VR, MINB, A>;
-    typename P::Acc acc[NC][NS][VR];
+    LapAcc<P, NC, NS, VR, A> acc[NC][NS][VR];
     // W~ of one site contiguous in visiting order (either vector layout)
     const E *inj = in + 2LL * j * VR;
     auto hop = [&](int q, const cx<A>(&Wm)[NC][NC]) {
