@@ -177,8 +177,11 @@ inline bool variant_ok(const dirac_op *op, int vr, int minb) {
 // D_W N_c = 2: 39 and 35 us, 4: 103 and 85 (N_c = 1: 14.9 and 16.0, N_c = 6,
 // N_v = 5: 109 and 117, left alone); D_S N_c = 2: 14 and 12, 4: 35 and 29, 6:
 // 119 and 111 (N_c = 1: 9.7 and 12.3); the Laplacian wlap N_c = 2: 39 and 36
-// (N_c = 4, VR = 1: 102 and 113), blap N_c = 4: 125 and 118 on 8^3x16, 6: 448
-// and 318 (N_c = 2: 47 and 49).
+// (N_c = 4, VR = 1: 102 and 113); blap N_c = 4: 125 and 118 on 8^3x16, and on
+// 12^3x16 N_c = 5, N_v = 6: 550 and 371 (N_c = 6: 565 and 661, left alone; N_c = 2:
+// 47 and 49); bsuv N_c = 6, N_v = 8: 370 and 310, N_v = 3: 369 and 431, 7: 552 and
+// 412 (N_c = 5, N_v = 8: 294 and 226, but N_v = 3: 261 and 313, 4: 217 and 237, 6:
+// 268 and 345, left alone).
 template <int NC, int NS, int VR, int MINB, typename A>
 constexpr int stencil_min_blocks(bool bound, int extra) {
     if (MINB > 1) return 1;

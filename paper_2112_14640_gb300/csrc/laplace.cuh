@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(stencil_max_threads(MINB),
 // thread reads its own.
 template <int NC, int NS, int VR, typename E, int MINB, int LAYOUT, bool STAGED>
 __global__ void __launch_bounds__(stencil_max_threads(MINB),
-                                  (stencil_min_blocks<NC, NS, VR, MINB, typename Acc<E>::T>(NC >= 4, NC * NS * VR + NC * NC)))
+                                  (stencil_min_blocks<NC, NS, VR, MINB, typename Acc<E>::T>(NS == 4 ? NC == 4 || NC == 5 : NC == 4 || NC >= 6, NC * NS * VR + NC * NC)))
     blap_kernel(const E *__restrict__ W, const E *__restrict__ in, E *__restrict__ out, Lat g,
                 typename Acc<E>::T centre) {
     using A = typename Acc<E>::T;
