@@ -305,8 +305,15 @@ int launch_laplace_v(const dirac_op *op, const void *in, void *out, double m, cu
                             return launch_check("wlap_kernel");
                         });
                     });
+                // read by each thread: FP64, bound by its own pipe (bsuv, 16^4,
+                // N_c = 3, N_v = 4: 1.53 ms, staged 1.58; blap 5.77 and 5.92); and
+                // N_c = 1 on site-inner vectors once four threads share the 8 bytes
+                // of a matrix (blap, 16^4, N_v = 8: 72 and 75 us, 12: 115 and 124, 24:
+                // 210 and 228; N_v = 4: 51 and 47; site-outer, N_v = 12: 152 and 140)
+                const bool direct = sizeof(E) == 8 || (NC == 1 && LAYOUT == DIRAC_LAYOUT_SITE_INNER && VR == 2 &&
+                                                       nchunk >= 4 && spins_of(op->kind) == 4);
                 const size_t smem = NC <= kMaxNcSmall ? wst::smem_bytes<NC, E>(block, nchunk) : 0;
-                if (NC > kMaxNcSmall || nchunk < wst::kMinChunks<E> || smem > wst::kMaxSmem)
+                if (NC > kMaxNcSmall || direct || nchunk < wst::kMinChunks<E> || smem > wst::kMaxSmem)
                     return on_spins([&](auto nsc) {
                         constexpr int NS = decltype(nsc)::value;
                         return run_w(blap_kernel<NC, NS, VR, E, 1, LAYOUT, false>,
