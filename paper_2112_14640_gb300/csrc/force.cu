@@ -63,37 +63,6 @@ __device__ __forceinline__ void add_outer(cx<A> (&M)[NC][NC], const cx<A> (&x)[N
             for (int b = 0; b < NC; ++b) cmac(M[a][b], x[a][v], conj(y[b][v]));
 }
 
-// (1 + a gamma_mu) applied to the 4 spin components p[0..3]
-template <typename A>
-__device__ __forceinline__ void apply_proj(int mu, A a, const cx<A> p[4], cx<A> q[4]) {
-    switch (mu) {
-    case 0:   // gamma_1 psi = (-i p3, -i p2, i p1, i p0)
-        q[0] = p[0] - a * times_i(p[3]);
-        q[1] = p[1] - a * times_i(p[2]);
-        q[2] = p[2] + a * times_i(p[1]);
-        q[3] = p[3] + a * times_i(p[0]);
-        break;
-    case 1:   // gamma_2 psi = (-p3, p2, p1, -p0)
-        q[0] = p[0] - a * p[3];
-        q[1] = p[1] + a * p[2];
-        q[2] = p[2] + a * p[1];
-        q[3] = p[3] - a * p[0];
-        break;
-    case 2:   // gamma_3 psi = (-i p2, i p3, i p0, -i p1)
-        q[0] = p[0] - a * times_i(p[2]);
-        q[1] = p[1] + a * times_i(p[3]);
-        q[2] = p[2] + a * times_i(p[0]);
-        q[3] = p[3] - a * times_i(p[1]);
-        break;
-    default:  // gamma_4 psi = (p2, p3, p0, p1)
-        q[0] = p[0] + a * p[2];
-        q[1] = p[1] + a * p[3];
-        q[2] = p[2] + a * p[0];
-        q[3] = p[3] + a * p[1];
-        break;
-    }
-}
-
 // F = P_TA(U B - C U^dag) (mode 0) or G = bc (B^dag + C) (mode 1) for link (n, mu)
 template <int NC, typename E, int LAYOUT>
 __device__ __forceinline__ void force_out(const E *__restrict__ U, E *__restrict__ out, const Lat &g, long long tid,
@@ -158,49 +127,138 @@ __global__ void __launch_bounds__(128, (NC == 3 && VR < 4 && sizeof(E) == 4 ? VR
     cx<A> B[NC][NC], C[NC][NC];
     for (int a = 0; a < NC; ++a)
         for (int b = 0; b < NC; ++b) B[a][b] = C[a][b] = cx<A>{0, 0};
-    if constexpr (NC <= kMaxNcSmall) {
 #pragma unroll 1
-        for (int v = 0; v < g.nv; v += VR) {
-            cx<A> x[NC][VR], y[NC][VR];
-            // B: (1 - gamma) psi(n+mu), (1 - gamma) chi(n); C: (1 + gamma) psi(n), (1 + gamma) chi(n+mu)
-            load_half<NC, VR, 0, E, A>(psi + om + 2 * v, csd, mu, true, x);
-            load_half<NC, VR, 0, E, A>(chi + on + 2 * v, csd, mu, true, y);
-            add_outer<NC, VR, A>(B, x, y);
-            load_half<NC, VR, 1, E, A>(psi + om + 2 * v, csd, mu, true, x);
-            load_half<NC, VR, 1, E, A>(chi + on + 2 * v, csd, mu, true, y);
-            add_outer<NC, VR, A>(B, x, y);
-            load_half<NC, VR, 0, E, A>(psi + on + 2 * v, csd, mu, false, x);
-            load_half<NC, VR, 0, E, A>(chi + om + 2 * v, csd, mu, false, y);
-            add_outer<NC, VR, A>(C, x, y);
-            load_half<NC, VR, 1, E, A>(psi + on + 2 * v, csd, mu, false, x);
-            load_half<NC, VR, 1, E, A>(chi + om + 2 * v, csd, mu, false, y);
-            add_outer<NC, VR, A>(C, x, y);
-        }
-    } else {   // accumulators beyond the register file: products one component at a time
-        for (int v = 0; v < g.nv; ++v) {
-            cx<A> pn[NC][4], pm[NC][4], qn[NC][4], qm[NC][4];
-            for (int a = 0; a < NC; ++a) {
-                cx<A> cn[4], cm[4];
-                for (int s = 0; s < 4; ++s) {
-                    const long long on = 2 * (L::vec(g, n, NC * 4, 0) + (long long)(a * 4 + s) * csd + v);
-                    const long long om = 2 * (L::vec(g, m, NC * 4, 0) + (long long)(a * 4 + s) * csd + v);
-                    pn[a][s] = ld1<E, A>(psi + on);
-                    pm[a][s] = ld1<E, A>(psi + om);
-                    cn[s] = ld1<E, A>(chi + on);
-                    cm[s] = ld1<E, A>(chi + om);
-                }
-                apply_proj<A>(mu, (A)-1, cn, qn[a]);   // (1 - gamma_mu) chi(n)
-                apply_proj<A>(mu, (A)1, cm, qm[a]);    // (1 + gamma_mu) chi(n+mu)
-            }
-            for (int a = 0; a < NC; ++a)
-                for (int b = 0; b < NC; ++b)
-                    for (int s = 0; s < 4; ++s) {
-                        cmac(B[a][b], pm[a][s], conj(qn[b][s]));
-                        cmac(C[a][b], pn[a][s], conj(qm[b][s]));
-                    }
-        }
+    for (int v = 0; v < g.nv; v += VR) {
+        cx<A> x[NC][VR], y[NC][VR];
+        // B: (1 - gamma) psi(n+mu), (1 - gamma) chi(n); C: (1 + gamma) psi(n), (1 + gamma) chi(n+mu)
+        load_half<NC, VR, 0, E, A>(psi + om + 2 * v, csd, mu, true, x);
+        load_half<NC, VR, 0, E, A>(chi + on + 2 * v, csd, mu, true, y);
+        add_outer<NC, VR, A>(B, x, y);
+        load_half<NC, VR, 1, E, A>(psi + om + 2 * v, csd, mu, true, x);
+        load_half<NC, VR, 1, E, A>(chi + on + 2 * v, csd, mu, true, y);
+        add_outer<NC, VR, A>(B, x, y);
+        load_half<NC, VR, 0, E, A>(psi + on + 2 * v, csd, mu, false, x);
+        load_half<NC, VR, 0, E, A>(chi + om + 2 * v, csd, mu, false, y);
+        add_outer<NC, VR, A>(C, x, y);
+        load_half<NC, VR, 1, E, A>(psi + on + 2 * v, csd, mu, false, x);
+        load_half<NC, VR, 1, E, A>(chi + om + 2 * v, csd, mu, false, y);
+        add_outer<NC, VR, A>(C, x, y);
     }
     force_out<NC, E, LAYOUT>(U, out, g, tid, n, mu, c, B, C, bc0, bc1, bc2, bc3, mode);
+}
+
+// D_W above N_c = 4, one thread per row a of a link's matrices: B and C of a
+// whole link do not fit a thread's registers, and accumulators left to local
+// memory are what the results must not hang on (with N_c^2 of them indexed in
+// rolled loops the first 16 bytes of B were not zero at N_c = 7 and 8).  A row
+// of both is 4 N_c reals and every index here is a compile-time one.  A thread
+// loads its own colour of psi and chi; the colours of chi meet in shared
+// memory, and so do the rows at the end: of B (for U B and B^dag), of U (for
+// C U^dag), of M = U B - C U^dag.  Neighbouring threads take the colours of a site-outer
+// vector, consecutive links of a site-inner one.
+constexpr int kRowLinks = 32;   // links per block
+template <int NC, int VR, typename E, int LAYOUT>
+__global__ void __launch_bounds__(kRowLinks * NC, sizeof(E) == 4 ? 2 : 1)
+    force_rows_kernel(const E *__restrict__ U, const E *__restrict__ psi, const E *__restrict__ chi,
+                      E *__restrict__ out, Lat g, int bc0, int bc1, int bc2, int bc3, int mode) {
+    using L = Layout<LAYOUT>;
+    using A = typename Acc<E>::T;
+    using Chi = cx<A>[4][NC][VR][kRowLinks + 1];   // the four projected components, [colour][RHS][link]
+    using Rows = cx<A>[NC][NC][kRowLinks + 1];
+    __shared__ __align__(16) unsigned char buf[2 * sizeof(Chi) > sizeof(Rows) ? 2 * sizeof(Chi) : sizeof(Rows)];
+    Chi *ys = reinterpret_cast<Chi *>(buf);        // two, used in turn
+    auto &rows = *reinterpret_cast<Rows *>(buf);   // a matrix per link
+    const int l = LAYOUT == 0 ? threadIdx.x / NC : threadIdx.x % kRowLinks;
+    const int a = LAYOUT == 0 ? threadIdx.x % NC : threadIdx.x / kRowLinks;
+    const long long own = (long long)blockIdx.x * kRowLinks + l;
+    const bool live = own < g.V * 4;
+    const long long tid = live ? own : g.V * 4 - 1;
+    const long long n = tid / 4;
+    const int mu = (int)(tid % 4);
+    const Coord c = site_coords(g, n);
+    const long long m = neighbour(g, n, c, mu, +1);
+    const long long csd = L::cs_stride(g);
+    const long long oa = 2 * (a * 4) * csd;
+    const long long on = 2 * L::vec(g, n, NC * 4, 0) + oa, om = 2 * L::vec(g, m, NC * 4, 0) + oa;
+    cx<A> B[NC], C[NC];
+#pragma unroll
+    for (int b = 0; b < NC; ++b) B[b] = C[b] = cx<A>{0, 0};
+#pragma unroll 1
+    for (int v = 0, half = 0; v < g.nv; v += VR, half ^= 1) {
+        // B: (1 - gamma) psi(n+mu), (1 - gamma) chi(n); C: (1 + gamma) psi(n), (1 + gamma) chi(n+mu)
+        cx<A> x[4][1][VR], y[4][1][VR];
+        load_half<1, VR, 0, E, A>(psi + om + 2 * v, csd, mu, true, x[0]);
+        load_half<1, VR, 1, E, A>(psi + om + 2 * v, csd, mu, true, x[1]);
+        load_half<1, VR, 0, E, A>(psi + on + 2 * v, csd, mu, false, x[2]);
+        load_half<1, VR, 1, E, A>(psi + on + 2 * v, csd, mu, false, x[3]);
+        load_half<1, VR, 0, E, A>(chi + on + 2 * v, csd, mu, true, y[0]);
+        load_half<1, VR, 1, E, A>(chi + on + 2 * v, csd, mu, true, y[1]);
+        load_half<1, VR, 0, E, A>(chi + om + 2 * v, csd, mu, false, y[2]);
+        load_half<1, VR, 1, E, A>(chi + om + 2 * v, csd, mu, false, y[3]);
+        Chi &yv = ys[half];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int i = 0; i < VR; ++i) yv[k][a][i][l] = y[k][0][i];
+        __syncthreads();   // also ends the reads of the other half, before the next trip writes to it
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int b = 0; b < NC; ++b)
+#pragma unroll
+                for (int i = 0; i < VR; ++i) cmac(k < 2 ? B[b] : C[b], x[k][0][i], conj(yv[k][b][i][l]));
+    }
+    auto exchange = [&](const cx<A> (&row)[NC]) {
+        __syncthreads();   // what was there has been read
+#pragma unroll
+        for (int b = 0; b < NC; ++b) rows[a][b][l] = row[b];
+        __syncthreads();
+    };
+    exchange(B);
+    E *o = out + 2 * ((tid * NC + a) * NC);
+    auto put = [&](int b, cx<A> f) {
+        if (live) store_cx<E, 1, A>(o + 2 * b, &f);
+    };
+    if (mode == 1) {   // G = bc (B^dag + C)
+        const int coord = mu == 0 ? c.x : mu == 1 ? c.y : mu == 2 ? c.z : c.t;
+        const int ext = mu == 0 ? g.nx : mu == 1 ? g.ny : mu == 2 ? g.nz : g.nt;
+        const int bcm = mu == 0 ? bc0 : mu == 1 ? bc1 : mu == 2 ? bc2 : bc3;
+        const A ph = (coord == ext - 1) ? (A)bcm : (A)1;
+#pragma unroll
+        for (int b = 0; b < NC; ++b) put(b, ph * (conj(rows[b][a][l]) + C[b]));
+        return;
+    }
+    // M = U B - C U^dag, row a; U the phased link
+    const E *link = U + 2 * L::template mat<NC>(g, n, 4, mu) + 2 * L::template mat_stride<NC>(g) * (a * NC);
+    cx<A> M[NC], u[NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+        u[k] = ld1<E, A>(link + 2 * L::template mat_stride<NC>(g) * k);
+        M[k] = cx<A>{0, 0};
+    }
+#pragma unroll
+    for (int k = 0; k < NC; ++k)
+#pragma unroll
+        for (int b = 0; b < NC; ++b) cmac(M[b], u[k], rows[k][b][l]);
+    exchange(u);
+#pragma unroll
+    for (int k = 0; k < NC; ++k)
+#pragma unroll
+        for (int b = 0; b < NC; ++b) {
+            const cx<A> w = rows[b][k][l];
+            cmac(M[b], C[k], cx<A>{-w.re, w.im});
+        }
+    exchange(M);
+    // P_TA(M) = (M - M^dag)/2 - tr(M - M^dag)/(2 Nc)
+    A trim = 0;
+#pragma unroll
+    for (int b = 0; b < NC; ++b) trim += rows[b][b][l].im;
+    trim /= (A)NC;
+#pragma unroll
+    for (int b = 0; b < NC; ++b) {
+        const cx<A> t = rows[b][a][l];
+        put(b, cx<A>{(A)0.5 * (M[b].re - t.re), (A)0.5 * (M[b].im + t.im) - (a == b ? trim : (A)0)});
+    }
 }
 
 template <int NC, int VR, typename E, int LAYOUT>
@@ -271,12 +329,16 @@ static int run_force(const dirac_op *op, const void *psi, const void *chi, void 
         const unsigned blocks = grid_for(op->V * 4, 128);
         const int *bc = op->geom.bc;
         const E *U = (const E *)op->links, *p = (const E *)psi, *c = (const E *)chi;
-        if (op->kind == DIRAC_STAGGERED)
-            force_stag_kernel<NC, VR, E, LAYOUT>
-                <<<blocks, 128, 0, s>>>(U, p, c, (E *)force_out, op->lat, bc[0], bc[1], bc[2], bc[3], mode);
-        else
+        if (op->kind == DIRAC_STAGGERED) {
+            if constexpr (NC <= kMaxNcSmall || VR == 1)
+                force_stag_kernel<NC, VR, E, LAYOUT>
+                    <<<blocks, 128, 0, s>>>(U, p, c, (E *)force_out, op->lat, bc[0], bc[1], bc[2], bc[3], mode);
+        } else if constexpr (NC <= kMaxNcSmall)
             force_kernel<NC, VR, E, LAYOUT>
                 <<<blocks, 128, 0, s>>>(U, p, c, (E *)force_out, op->lat, bc[0], bc[1], bc[2], bc[3], mode);
+        else
+            force_rows_kernel<NC, VR, E, LAYOUT><<<grid_for(op->V * 4, kRowLinks), kRowLinks * NC, 0, s>>>(
+                U, p, c, (E *)force_out, op->lat, bc[0], bc[1], bc[2], bc[3], mode);
         return launch_check(op->kind == DIRAC_STAGGERED ? "force_stag_kernel" : "force_kernel");
     });
 }
@@ -301,7 +363,8 @@ extern "C" int dirac_force(const dirac_op *op, const void *psi, const void *chi,
     // (D_S with fewer than eight: two trips of half the width overlap better)
     int vr = op->prec == DIRAC_F32 && (op->kind == DIRAC_WILSON || op->nv >= 8) ? 4 : 2;
     while (op->nv % vr) vr /= 2;
-    vr = op->nc > kMaxNcSmall ? 1 : aligned_vr(vr, op->prec, psi, chi);
+    vr = aligned_vr(vr, op->prec, psi, chi);
+    if (op->nc > kMaxNcSmall) vr = op->kind == DIRAC_WILSON && op->prec == DIRAC_F32 && op->nv % 2 == 0 ? 2 : 1;
     return dispatch_prec(op->prec, [&](auto tag) {
         using E = std::remove_pointer_t<decltype(tag)>;
         if constexpr (sizeof(E) == 2) {
@@ -312,6 +375,8 @@ extern "C" int dirac_force(const dirac_op *op, const void *psi, const void *chi,
                 if constexpr (NC <= kMaxNcSmall) {
                     if constexpr (sizeof(E) == 4)
                         if (vr == 4) return run_force<NC, 4, E>(op, psi, chi, force_out, mode, s);
+                    if (vr == 2) return run_force<NC, 2, E>(op, psi, chi, force_out, mode, s);
+                } else if constexpr (sizeof(E) == 4) {
                     if (vr == 2) return run_force<NC, 2, E>(op, psi, chi, force_out, mode, s);
                 }
                 return run_force<NC, 1, E>(op, psi, chi, force_out, mode, s);

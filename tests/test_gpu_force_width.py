@@ -1,6 +1,6 @@
 """The D_W and D_S force against the oracle at every number of right-hand sides
 a load can take (1, 2, 4 and remainders), on vectors that start on a 16-byte but
-not a 32-byte boundary, and at N_c 1..6.  Tolerance: a component is a sum of
+not a 32-byte boundary, and at N_c 1..8.  Tolerance: a component is a sum of
 8 N_v products (N_v = 12: 96) of rounded inputs, FP32 unit roundoff 6e-8: 1e-5."""
 import numpy as np
 import pytest
@@ -27,7 +27,8 @@ def shifted(v):
 
 
 @pytest.mark.parametrize("kind", [D.WILSON, D.STAGGERED])
-@pytest.mark.parametrize("nc,nv", [(3, 1), (3, 2), (3, 6), (3, 8), (3, 12), (1, 4), (2, 8), (4, 4), (4, 2), (5, 4), (6, 2)])
+@pytest.mark.parametrize("nc,nv", [(3, 1), (3, 2), (3, 6), (3, 8), (3, 12), (1, 4), (2, 8), (4, 4), (4, 2), (5, 4), (6, 2), (7, 2),
+                                   (8, 1), (8, 3)])
 def test_force_widths(kind, nc, nv):
     dims = (2, 4, 2, 6)
     U = I.gauge_field(dims, nc, 0.4, 71)
