@@ -409,6 +409,25 @@ __device__ __forceinline__ const double *last_block_sum(const RedRow<A> *partial
     return sums;
 }
 
+// The rows row, row + stride, ... of a thread, four at a time: batch(count,
+// whole, row) takes `count` of them and skips those past the end unless
+// `whole`.  Four complex numbers per access (16-bit storage) unpack to twice the
+// registers that two FP32 ones take: with the skips the four rows are held at
+// once (update 154 registers, one block per SM), so there whole batches are
+// followed by single rows (48 registers; 32^3x16, N_v = 12, FP16: update 419 and
+// 228 us, a memory rate of 6.6 TB/s).  Elsewhere the single rows at the end cost
+// more (8^4, N_v = 3: 3.90 and 3.98 ms a solve).
+template <int G, typename BATCH>
+__device__ __forceinline__ void rows_by_four(long long row, long long stride, long long rows, BATCH batch) {
+    using Four = std::integral_constant<int, 4>;
+    if constexpr (G == 4) {
+        for (; row + 3 * stride < rows; row += 4 * stride) batch(Four{}, std::true_type{}, row);
+        for (; row < rows; row += stride) batch(std::integral_constant<int, 1>{}, std::true_type{}, row);
+    } else {
+        for (; row < rows; row += 4 * stride) batch(Four{}, std::false_type{}, row);
+    }
+}
+
 __device__ __forceinline__ bool cg_stopped(const CgScalars &k) { return k.ctl && *(volatile int *)k.ctl; }
 
 template <typename E, int G>
@@ -427,20 +446,21 @@ __global__ void cg_dot_kernel(const E *__restrict__ x, const E *__restrict__ y, 
         }
     };
     if (live)
-        for (long long row = (long long)blockIdx.x * R + r; row < rows; row += 4 * stride) {
-            cx<A> a[4][G], b[4][G];
+        rows_by_four<G>((long long)blockIdx.x * R + r, stride, rows, [&](auto count, auto whole, long long row) {
+            constexpr int N = decltype(count)::value;
+            cx<A> a[N][G], b[N][G];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < N; ++u) {
                 const long long e = 2 * ((row + u * stride) * nv + vg * G);
-                if (row + u * stride < rows) {
+                if (whole || row + u * stride < rows) {
                     load_cx<E, G, A>(x + e, a[u]);
                     load_cx<E, G, A>(y + e, b[u]);
                 }
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (row + u * stride < rows) add(a[u], b[u]);
-        }
+            for (int u = 0; u < N; ++u)
+                if (whole || row + u * stride < rows) add(a[u], b[u]);
+        });
     RedRow<A> *partial = reinterpret_cast<RedRow<A> *>(k.partial);
     block_reduce(acc, sh, r, vg, R, ng,
                  [&](int c, const RedRow<A> &v) { partial[(long long)blockIdx.x * nv + c] = v; });
@@ -480,20 +500,22 @@ __global__ void cg_residual_kernel(E *rv, const E *__restrict__ q, long long row
         store_cx<E, G, A>(rv + e, o);
     };
     if (live)
-        for (long long row = (long long)blockIdx.x * R + r; row < rows; row += 4 * stride) {
-            cx<A> tr[4][G], tq[4][G];
+        rows_by_four<G>((long long)blockIdx.x * R + r, stride, rows, [&](auto count, auto whole, long long row) {
+            constexpr int N = decltype(count)::value;
+            cx<A> tr[N][G], tq[N][G];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < N; ++u) {
                 const long long e = 2 * ((row + u * stride) * nv + vg * G);
-                if (row + u * stride < rows) {
+                if (whole || row + u * stride < rows) {
                     load_cx<E, G, A>(rv + e, tr[u]);
                     load_cx<E, G, A>(q + e, tq[u]);
                 }
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (row + u * stride < rows) finish(2 * ((row + u * stride) * nv + vg * G), tr[u], tq[u]);
-        }
+            for (int u = 0; u < N; ++u)
+                if (whole || row + u * stride < rows)
+                    finish(2 * ((row + u * stride) * nv + vg * G), tr[u], tq[u]);
+        });
     RedRow<A> *partial = reinterpret_cast<RedRow<A> *>(k.partial);
     block_reduce(acc, sh, r, vg, R, ng,
                  [&](int c, const RedRow<A> &v) { partial[(long long)blockIdx.x * nv + c] = v; });
@@ -564,21 +586,23 @@ __global__ void cg_update_kernel(E *x, E *p, const E *__restrict__ r_, long long
         store_cx<E, G, A>(x + e, xv);
         store_cx<E, G, A>(p + e, pv);
     };
-    for (long long row = (long long)blockIdx.x * R + r; row < rows; row += 4 * stride) {
-        cx<A> xv[4][G], pv[4][G], rv[4][G];
+    rows_by_four<G>((long long)blockIdx.x * R + r, stride, rows, [&](auto count, auto whole, long long row) {
+        constexpr int N = decltype(count)::value;
+        cx<A> xv[N][G], pv[N][G], rv[N][G];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < N; ++u) {
             const long long e = 2 * ((row + u * stride) * nv + vg * G);
-            if (row + u * stride < rows) {
+            if (whole || row + u * stride < rows) {
                 load_cx<E, G, A>(x + e, xv[u]);
                 load_cx<E, G, A>(p + e, pv[u]);
                 load_cx<E, G, A>(r_ + e, rv[u]);
             }
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (row + u * stride < rows) finish(2 * ((row + u * stride) * nv + vg * G), xv[u], pv[u], rv[u]);
-    }
+        for (int u = 0; u < N; ++u)
+            if (whole || row + u * stride < rows)
+                finish(2 * ((row + u * stride) * nv + vg * G), xv[u], pv[u], rv[u]);
+    });
 }
 
 #undef BLAS_THREAD_SETUP
