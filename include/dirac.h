@@ -271,7 +271,8 @@ int dirac_halo_unpack(const dirac_op *op, const void *buf, int t, int proj, void
  * resident 128-thread blocks per SM (1 = the compiler's choice; 3, 4, 5, 6
  * compiled for N_c = 3 only); block = threads per block, a multiple of 32 up
  * to 128 minb (0 = 128).  vr = 0 restores the default choice (which for FP64
- * on small lattices is a kernel without variants).  Errors:
+ * on small lattices is a kernel without variants).  Solves in the operator's
+ * own precision iterate with the variant too, in whichever layout.  Errors:
  * DIRAC_ERR_INVALID_ARG for a variant that is not compiled, a vr that does
  * not divide N_v or a block size out of range. */
 int dirac_op_set_launch(dirac_op *op, int vr, int minb, int block);
@@ -279,9 +280,10 @@ int dirac_op_get_launch(const dirac_op *op, int *vr, int *minb, int *block);
 /* Time every compiled variant of D (bare mass m0) on operator-owned buffers
  * and keep the fastest for this operator; the choice is also remembered for
  * operators created later in this process with the same kind, layout,
- * precision, link storage, N_c, N_v and volume (including what the solvers
- * iterate with: the site-inner form of the operator, and the site-inner
- * lower-precision twin of a mixed solve).
+ * precision, link storage, N_c, N_v and volume.  The solvers iterate on
+ * site-inner vectors: with what was tuned for the site-inner form of the
+ * operator (of the lower-precision twin in a mixed solve), else with what was
+ * tuned for the site-outer one.
  * best_ms (may be NULL) receives the winner's time per apply.  Synchronises. */
 int dirac_op_autotune(dirac_op *op, double m0, void *stream, double *best_ms);
 

@@ -154,24 +154,26 @@ struct TuneVal {
 static std::mutex g_tune_mu;
 static std::map<TuneKey, TuneVal> g_tune;
 
-static TuneKey tune_key(const dirac_op *op) {
-    return TuneKey{(int)op->kind, op->geom.layout, (int)op->prec, (int)link_prec(op), op->nc, op->nv, op->V,
+static TuneKey tune_key(const dirac_op *op, int layout) {
+    return TuneKey{(int)op->kind, layout, (int)op->prec, (int)link_prec(op), op->nc, op->nv, op->V,
                    op->clover != nullptr};
 }
 
 static void remember_tuning(const dirac_op *op) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    g_tune[tune_key(op)] = TuneVal{op->vr, op->minb, op->block};
+    g_tune[tune_key(op, op->geom.layout)] = TuneVal{op->vr, op->minb, op->block};
 }
 
-static void recall_tuning(dirac_op *op) {
+// The variant remembered for op's shape on vectors of `layout`, if any.
+static bool recall_tuning(dirac_op *op, int layout) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    auto it = g_tune.find(tune_key(op));
-    if (it != g_tune.end()) {
-        op->vr = it->second.vr;
-        op->minb = it->second.minb;
-        op->block = it->second.block;
-    }
+    auto it = g_tune.find(tune_key(op, layout));
+    if (it == g_tune.end()) return false;
+    op->vr = it->second.vr;
+    op->minb = it->second.minb;
+    op->block = it->second.block;
+    op->variant_set = false;
+    return true;
 }
 
 // Allocate an operator handle of the given geometry without links.
@@ -201,19 +203,20 @@ int op_alloc(dirac_kind kind, const dirac_geom *g, dirac_op **out) {
         op_free(op);
         return rc;
     }
-    recall_tuning(op);
+    recall_tuning(op, g->layout);
     *out = op;
     return DIRAC_OK;
 }
 
 // Links, W and clover blocks are stored alike for both vector layouts, so the
-// view needs no copies; it launches with what was tuned for its own layout.
+// view needs no copies.  It launches with the variant the caller set for op;
+// else with what was tuned for site-inner vectors; else with what was tuned
+// for op's own (every variant is compiled for both layouts).
 dirac_op op_site_inner(const dirac_op *op) {
     dirac_op view = *op;
     if (op->geom.layout != DIRAC_LAYOUT_SITE_INNER) {
         view.geom.layout = DIRAC_LAYOUT_SITE_INNER;
-        view.vr = view.minb = view.block = 0;
-        recall_tuning(&view);
+        if (!op->variant_set) recall_tuning(&view, DIRAC_LAYOUT_SITE_INNER);
     }
     return view;
 }
@@ -239,6 +242,9 @@ int op_inner(const dirac_op *op, dirac_prec p, int link_storage, dirac_op **out,
             tw->csw = op->csw;
             rc = alloc(&tw->clover, tw->link_bytes);
         }
+        // tuned for site-inner vectors (the key knows of the clover term now),
+        // else for the caller's layout
+        if (!recall_tuning(tw, DIRAC_LAYOUT_SITE_INNER) && !tw->vr) recall_tuning(tw, op->geom.layout);
         if (!rc) rc = launch_convert_links(op, tw, s);
         if (rc) {
             op_free(tw);
@@ -324,7 +330,7 @@ int dirac_op_set_clover(dirac_op *op, double csw, const void *V, dirac_prec v_pr
         cudaFree(op->clover);
         op->clover = nullptr;
         op->csw = 0.0;
-        recall_tuning(op);
+        recall_tuning(op, op->geom.layout);
         return rc;
     }
     int rc = op->clover ? DIRAC_OK : alloc(&op->clover, op->link_bytes);
@@ -337,7 +343,7 @@ int dirac_op_set_clover(dirac_op *op, double csw, const void *V, dirac_prec v_pr
         op->clover = nullptr;
         op->csw = 0.0;
     }
-    recall_tuning(op);
+    recall_tuning(op, op->geom.layout);
     return rc;
 }
 
@@ -407,6 +413,7 @@ int dirac_op_set_launch(dirac_op *op, int vr, int minb, int block) {
     if (!op) return DIRAC_ERR_INVALID_ARG;
     if (vr == 0) {
         op->vr = op->minb = op->block = 0;
+        op->variant_set = false;
         return DIRAC_OK;
     }
     if (!variant_ok(op, vr, minb)) return DIRAC_ERR_INVALID_ARG;
@@ -415,6 +422,7 @@ int dirac_op_set_launch(dirac_op *op, int vr, int minb, int block) {
     op->vr = vr;
     op->minb = minb;
     op->block = block;
+    op->variant_set = true;
     return DIRAC_OK;
 }
 
@@ -485,6 +493,7 @@ int dirac_op_autotune(dirac_op *op, double m0, void *stream, double *best_ms) {
     op->vr = best->vr;
     op->minb = best->minb;
     op->block = best->block;
+    op->variant_set = false;
     remember_tuning(op);
     if (best_ms) *best_ms = best->ms;
     return DIRAC_OK;

@@ -40,6 +40,7 @@ struct dirac_op {
     dirac_op *inner[4][2]; // lower-precision twins for mixed solves (lazy), by [prec][link storage]
     int vr, minb, block;   // stencil launch variant (RHS per thread, register class, threads per block);
                            // 0 = default
+    bool variant_set;      // the variant is the caller's own (dirac_op_set_launch), not a tuned one
 };
 
 namespace dgb {
