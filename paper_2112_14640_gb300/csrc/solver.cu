@@ -302,7 +302,10 @@ int solver_cg_step(const dirac_op *op, const void *p, void *q, double m0, const 
 struct CgRun {
     int done = 0;                  // iterations the device carried out
     const double *hist = nullptr;  // done x (pq, old rr, new rr) x nv
-    double log_rate = -0.5;        // last seen change of log |r|^2 per iteration (slowest RHS)
+    double log_rate[kNS];          // last seen change of log |r|^2 per iteration, per RHS
+    CgRun() {
+        for (double &r : log_rate) r = -0.5;
+    }
 };
 
 // Largest vector whose iterations go through a graph: above it an iteration
@@ -311,13 +314,19 @@ constexpr size_t kCgGraphBytes = 32u << 20;
 
 // How many iterations to enqueue before the host looks again.  The launches of
 // iterations past the stop rule cost little (their vector passes return at
-// once) but their stencils run, so the run stays short of where the residual
-// is predicted to pass: `need` = log of the drop in |r|^2 still missing.
-static int run_length(const CgRun &run, double need) {
-    double n = need / run.log_rate;   // both negative
-    if (!(n > 0)) n = 1;
+// once) but their stencils run, so the run stays short of where the rule is
+// predicted to be met: need[v] = log of the drop in |r|^2 that RHS v still
+// misses, and the rule waits for every active RHS, or for the first of them
+// (`any`).  Frozen RHS do not count.
+static int run_length(const CgRun &run, int nv, const double *act, const double *need, bool any) {
+    double n = any ? 1e300 : 0;
+    for (int v = 0; v < nv; ++v) {
+        if (act[v] == 0.0) continue;
+        const double m = need[v] / run.log_rate[v];   // both negative
+        n = any ? fmin(n, m) : fmax(n, m);
+    }
     n *= 0.7;
-    return n < 1 ? 1 : n > kCgHistory ? kCgHistory : (int)n;
+    return !(n >= 1) ? 1 : n > kCgHistory ? kCgHistory : (int)n;
 }
 
 // The launches of one iteration: the update of x and p that the one before
@@ -381,12 +390,11 @@ static int cg_run(const dirac_op *op, void *r, void *pv, void *q, void *x, doubl
     run.done = ((const int *)op->solver_host)[1];
     run.hist = op->solver_host + 2;
     if (run.done < 1 || run.done > n) return DIRAC_ERR_CUDA;   // the launches did not run
-    double rate = -1e300;
     for (int v = 0; v < nv; ++v) {
         const double first = run.hist[nv + v], last = run.hist[((run.done - 1) * 3 + 2) * nv + v];
-        if (first > 0 && last > 0) rate = fmax(rate, log(last / first) / run.done);
+        const double rate = first > 0 && last > 0 ? log(last / first) / run.done : 0.0;
+        if (rate < -1e-3) run.log_rate[v] = rate;
     }
-    if (rate > -1e300 && rate < -1e-3) run.log_rate = rate;
     return DIRAC_OK;
 }
 
@@ -398,7 +406,7 @@ static int cg_core(const dirac_op *op, const void *rhs, void *x, double m0, doub
     const int nv = op->nv;
     const dirac_prec p = op->prec;
     void *r = w.v[0], *pv = w.v[1], *q = w.v[2];
-    double nb[kNS], rr[kNS], act[kNS], rrt[kNS];
+    double nb[kNS], rr[kNS], act[kNS], rrt[kNS], need[kNS];
     TRY(cuda_check(cudaMemsetAsync(w.counter, 0, sizeof(unsigned), s), "reduction counter"));
     TRY(blas_norm2(op, p, rhs, w.nb, s));
     // r = rhs - A x
@@ -408,14 +416,13 @@ static int cg_core(const dirac_op *op, const void *rhs, void *x, double m0, doub
     TRY(to_host(nb, w.nb, nv, s));
     TRY(to_host(rr, w.rr, nv, s));
     int nact = 0;
-    double need = 0;
     for (int v = 0; v < nv; ++v) {
         const bool conv = nb[v] == 0.0 || sqrt(rr[v]) < tol * sqrt(nb[v]);
         act[v] = conv ? 0.0 : 1.0;
         out.status_rhs[v] = conv ? DIRAC_OK : DIRAC_NOT_CONVERGED;
         out.relres[v] = nb[v] > 0 ? sqrt(rr[v] / nb[v]) : 0.0;
         nact += !conv;
-        if (!conv) need = fmin(need, log(tol * tol * nb[v] / rr[v]));
+        need[v] = log(tol * tol * nb[v] / rr[v]);
     }
     TRY(to_dev(w.act, act, nv, s));
     CgScalars c = cg_scalars(w);
@@ -429,7 +436,7 @@ static int cg_core(const dirac_op *op, const void *rhs, void *x, double m0, doub
     out.status = DIRAC_OK;
     int it = 0;
     while (nact > 0) {
-        int n = run_length(run, need);
+        int n = run_length(run, nv, act, need, false);
         if (it == 0 && n > 4) n = 4;   // no rate seen yet
         n = n < every - it % every ? n : every - it % every;
         n = n < maxit - it ? n : maxit - it;
@@ -442,13 +449,10 @@ static int cg_core(const dirac_op *op, const void *rhs, void *x, double m0, doub
         it += run.done;
         const double *rn = run.hist + ((run.done - 1) * 3 + 2) * nv;
         bool all_pass = true, finite = true;
-        need = 0;
         for (int v = 0; v < nv; ++v) {
             if (!isfinite(rn[v])) finite = false;
-            if (act[v] != 0.0 && !(sqrt(rn[v]) < tol * sqrt(nb[v]))) {
-                all_pass = false;
-                need = fmin(need, log(tol * tol * nb[v] / rn[v]));
-            }
+            if (act[v] != 0.0 && !(sqrt(rn[v]) < tol * sqrt(nb[v]))) all_pass = false;
+            need[v] = log(tol * tol * nb[v] / rn[v]);
         }
         if (!finite) {
             out.status = DIRAC_NONFINITE;
@@ -462,7 +466,6 @@ static int cg_core(const dirac_op *op, const void *rhs, void *x, double m0, doub
             TRY(to_host(rrt, w.rr_new, nv, s));
             bool stagnated = false, froze = false;
             nact = 0;
-            need = 0;
             for (int v = 0; v < nv; ++v) {
                 out.relres[v] = nb[v] > 0 ? sqrt(rrt[v] / nb[v]) : 0.0;
                 if (act[v] == 0.0) continue;
@@ -474,7 +477,7 @@ static int cg_core(const dirac_op *op, const void *rhs, void *x, double m0, doub
                 }
                 const double disc = fabs(sqrt(rn[v]) - sqrt(rrt[v])) / fmax(sqrt(rrt[v]), 1e-300);
                 if (disc > 0.01) stagnated = true;
-                need = fmin(need, log(tol * tol * nb[v] / rrt[v]));
+                need[v] = log(tol * tol * nb[v] / rrt[v]);
                 ++nact;
             }
             if (froze) TRY(to_dev(w.act, act, nv, s));
@@ -712,11 +715,12 @@ static int cg_reliable(const dirac_op *hi, const dirac_op *lo, const void *rhs, 
     CgRun run;
     CgGraph graph;
     TRY(cuda_check(cudaMemsetAsync(wl.run, 0, 2 * sizeof(double), s), "run control"));
-    double need = -1;
+    double need[kNS];
+    for (double &d : need) d = -1;
     out.status = DIRAC_OK;
     int it = 0;
     while (nact > 0) {
-        int n = run_length(run, need);
+        int n = run_length(run, nv, act, need, true);
         if (it == 0 && n > 4) n = 4;   // no rate seen yet
         n = n < maxit - it ? n : maxit - it;
         TRY(cg_run(lo, rs, ps, qs, ys, m0, n, c, wl, run, graph, s));
@@ -746,10 +750,9 @@ static int cg_reliable(const dirac_op *hi, const dirac_op *lo, const void *rhs, 
                 for (int v = 0; v < nv; ++v) rmax[v] = fmax(rmax[v], sqrt(rk[v]));
         }
         double rn[kNS];
-        need = -1e300;
         for (int v = 0; v < nv; ++v) {
             rn[v] = rn_dev[v];
-            if (act[v] != 0.0 && rn[v] > 0) need = fmax(need, goal[v] - log(rn[v]));
+            need[v] = goal[v] - log(rn[v]);
         }
         if (!finite) {
             out.status = DIRAC_NONFINITE;
@@ -828,9 +831,7 @@ static int cg_reliable(const dirac_op *hi, const dirac_op *lo, const void *rhs, 
                 sig_h[v] = (act[v] != 0.0 && rrt[v] > 0) ? unit / sqrt(rrt[v]) : 0.0;
             }
             TRY(upload());
-            need = -1e300;
-            for (int v = 0; v < nv; ++v)
-                if (act[v] != 0.0 && rn[v] > 0) need = fmax(need, goal[v] - log(rn[v]));
+            for (int v = 0; v < nv; ++v) need[v] = goal[v] - log(rn[v]);
             TRY(solver_cg_beta(lo, wl.rr_new, c, s));
             TRY(blas_axpby(lo, pl, ps, rs, nullptr, 1.0, ps, wl.beta, 1.0, nullptr, s));
             TRY(cuda_check(cudaMemsetAsync(wl.run, 0, 2 * sizeof(double), s), "run control"));   // nothing due
