@@ -245,9 +245,12 @@ inline void launch_variant(const dirac_op *op, int &vr, int &minb, int &block) {
     if (op->kind == DIRAC_STAGGERED && op->prec == DIRAC_F32 && op->nc <= kMaxNcSmall && op->nv % 4 == 0 &&
         op->V * op->nv / 4 >= 2 * 608 * 32)
         vr = 4;
+    // D_S classes: 16^3x32, N_v = 8, BF16 23.1 us with FP32 links in class 3 (24.8 in
+    // 5), 24.9 with BF16 links in class 5 (26.9 in 3); FP64 takes the same time in
+    // 6 as in 3 (16^4, N_v = 1 to 12)
     if (op->nc == 3) {
         if (op->kind == DIRAC_WILSON) minb = vr == 4 ? 3 : 4;
-        else if (op->kind == DIRAC_STAGGERED) minb = vr == 4 ? 5 : 6;
+        else if (op->kind == DIRAC_STAGGERED) minb = vr == 4 ? (link_prec(op) != op->prec ? 3 : 5) : 6;
     }
     // 81-point stencils on 4 spins in FP32 arithmetic: two accumulators per
     // component (common.cuh), so one RHS per thread from N_c = 3 on (16^3x32,
