@@ -155,7 +155,10 @@ __global__ void __launch_bounds__(128, (NC == 3 && VR < 4 && sizeof(E) == 4 ? VR
 // loads its own colour of psi and chi; the colours of chi meet in shared
 // memory, and so do the rows at the end: of B (for U B and B^dag), of U (for
 // C U^dag), of M = U B - C U^dag.  Neighbouring threads take the colours of a site-outer
-// vector, consecutive links of a site-inner one.
+// vector, consecutive links of a site-inner one.  A thread per link before and
+// now, us, 12^3x16, FP32, N_v = 4, site-inner: N_c = 5 78 and 66, 6 165 and 91, 7
+// 325 and 112, 8 413 and 154 (every colour's chi read by every row: 135 at
+// N_c = 5); 8^3x16, FP64, N_v = 2: 220 and 133, 345 and 197, 431 and 292, 592 and 401.
 constexpr int kRowLinks = 32;   // links per block
 template <int NC, int VR, typename E, int LAYOUT>
 __global__ void __launch_bounds__(kRowLinks * NC, sizeof(E) == 4 ? 2 : 1)
@@ -359,9 +362,15 @@ extern "C" int dirac_force(const dirac_op *op, const void *psi, const void *chi,
     cudaStream_t s = (cudaStream_t)stream;
     // the handle owns the Brillouin force's scratch (allocated on first use)
     if (op->kind == DIRAC_BRILLOUIN) return launch_bril_force(const_cast<dirac_op *>(op), psi, chi, force_out, mode, s);
-    // right-hand sides per load: 32 bytes where N_v and the vectors allow
-    // (D_S with fewer than eight: two trips of half the width overlap better)
-    int vr = op->prec == DIRAC_F32 && (op->kind == DIRAC_WILSON || op->nv >= 8) ? 4 : 2;
+    // right-hand sides per load: 32 bytes where N_v and the vectors allow.  D_S
+    // with fewer than eight: two trips of half the width overlap better (16^3x32,
+    // N_v = 4, site-inner, N_c = 3: 48 us, one trip 54; N_c = 2: 22.7 and 20.6, so
+    // not there).  D_W on site-inner vectors at N_c = 1, 2, where the loads of a
+    // warp are whole lines anyway: one each up to N_v = 4 (25 and 57 us, four: 29
+    // and 62; N_v = 8: 88 and 178, four: 52 and 99).
+    const bool narrow = op->kind == DIRAC_WILSON && op->geom.layout == DIRAC_LAYOUT_SITE_INNER && op->nc <= 2 &&
+                        op->nv <= 4 && op->prec == DIRAC_F32;
+    int vr = narrow ? 1 : op->prec == DIRAC_F32 && (op->kind == DIRAC_WILSON || op->nv >= 8 || op->nc <= 2) ? 4 : 2;
     while (op->nv % vr) vr /= 2;
     vr = aligned_vr(vr, op->prec, psi, chi);
     if (op->nc > kMaxNcSmall) vr = op->kind == DIRAC_WILSON && op->prec == DIRAC_F32 && op->nv % 2 == 0 ? 2 : 1;
