@@ -1,6 +1,7 @@
 """The 81-point stencils around the line between the two ways they read W~: a
-block's ring in shared memory from four threads per site on, each thread's own
-loads below.  Odd volumes leave a ragged last block whose idle threads still
+block's ring in shared memory wherever it fits, or each thread's own loads (one
+right-hand side at N_c = 3 and 4; FP64 Laplacians; FP64 D_B with fewer than four
+threads per site; N_c = 1 Laplacians on site-inner vectors).  Odd volumes leave a ragged last block whose idle threads still
 take part in the copies; extent 2 wraps every offset."""
 import numpy as np
 import pytest
@@ -17,6 +18,7 @@ BC = (1, 1, -1, -1)
 
 
 @pytest.mark.parametrize("nc,nv,prec,links", [
+    (3, 1, D.F32, 0), (4, 1, D.F32, 0), (3, 1, D.F64, 0), (1, 8, D.F32, 0), (1, 24, D.F32, 0),
     (3, 3, D.F32, 0), (3, 4, D.F32, 0), (3, 7, D.F32, 0), (3, 8, D.F64, 0), (3, 64, D.F32, 0), (1, 5, D.F32, 0),
     (2, 6, D.F64, 0), (4, 4, D.F32, 0), (4, 5, D.F64, 0), (1, 16, D.BF16, 0), (2, 9, D.F16, 0), (3, 12, D.BF16, 0),
     (3, 16, D.F16, 1), (4, 8, D.F16, 0)])
