@@ -356,9 +356,9 @@ __global__ void axpby_kernel(E *z, const E *x, const E *y, const double *__restr
 // three, and no value the host has to see before the next launch.  The
 // iterations that the host enqueues ahead of the stop rule do nothing once it
 // has been met (ctl[0]).  Memory-bound on large lattices (16^3x32, D_W,
-// N_v = 4, FP32: dot 16, residual 26, update 42 us; the update moves 250 MB at
-// 6 TB/s), bound by the chain load - reduce - last block on small ones (8^4,
-// N_v = 3: about 5, 6 and 3 us).
+// N_v = 4, FP32, from cold caches: dot 23, residual 27, update 37 us; the update
+// moves 250 MB at 6.8 TB/s), bound by the chain load - reduce - last block on
+// small ones (8^4, N_v = 3: 8, 10 and 4 us).
 
 // Join the blocks' rows (nv sums each) in the last block to arrive; the N_v
 // values there, null in every other block.  Fixed order, so reproducible.

@@ -27,7 +27,7 @@ struct Offset {
     unsigned char prev[4];   // position in this table of s - s_mu mu (0 when that is the centre)
     // the offsets s +- mu one level up, for the 4 - k axes s does not move
     // along: axis, sign and position in this table
-    unsigned char nchild, cmu[6], child[6];
+    unsigned char cmu[6], child[6];
     signed char csign[6];
 };
 struct Table {
@@ -73,7 +73,6 @@ __host__ __device__ constexpr Table make_table() {
                 o.csign[c] = (signed char)sg;
                 o.child[c++] = (unsigned char)t.pos[d + sg * pow3[mu]];
             }
-        o.nchild = (unsigned char)c;
     }
     return t;
 }

@@ -255,7 +255,13 @@ inline void launch_variant(const dirac_op *op, int &vr, int &minb, int &block) {
     // 81-point stencils on 4 spins in FP32 arithmetic: two accumulators per
     // component (common.cuh), so one RHS per thread from N_c = 3 on (16^3x32,
     // N_v = 12, D_B: 1.07 ms, two RHS 1.06 ms at 8 warps per SM; the Brillouin
-    // Laplacian 0.94 against 1.13 ms)
+    // Laplacian 0.94 against 1.13 ms).  16-bit vectors too: their loads shrink to
+    // 4 bytes, but four RHS per thread, as before, took longer everywhere (16^4,
+    // FP16, N_v = 4: 250 and 534 us, 12: 705 and 970; with FP32 links 623 and 1344).
+    // FP64 keeps one RHS per thread in the compiler's own registers (in 384-thread
+    // blocks of class 3, as before, 16^4, N_c = 3, N_v = 1: 3.17 ms, now 2.13; 4: 7.91
+    // and 7.43; 12: 22.1 and 21.6; N_c = 4 had this form before and loses 3% below
+    // N_v = 12 by the row order: 12^3x16, N_v = 4: 5.18 and 5.35)
     if (uses_w(op->kind) && spins_of(op->kind) == 4 && op->prec != DIRAC_F64 && op->nc <= kMaxNcSmall) {
         vr = op->nc >= 3 || vr == 1 ? 1 : 2;
         if (op->nc == 3) minb = 4;

@@ -11,10 +11,10 @@
 // Laplacian reads the operator's stored W~_q = rho_k s_lead W_s (bril_dirs.h),
 // per site in visiting order, and weighs each with -c_k s_lead, which is
 // -lambda_k/2 on W_s; offsets and weights come from a table in constant
-// memory (one broadcast read per offset, uniform over the warp).  W~ is staged
-// in shared memory for the block (wstage.cuh) and its products are packed
-// (common.cuh): blap 0.991 -> 0.946 ms, bsuv 0.490 -> 0.313 ms at 16^3x32,
-// N_v = 12, N_c = 3, FP32.
+// memory (one broadcast read per offset, uniform over the warp).  In FP32 W~ is
+// staged in shared memory for the block (wstage.cuh) and its products are packed
+// (common.cuh): blap 0.991 -> 0.920 ms, bsuv 0.490 -> 0.293 ms at 16^3x32,
+// N_v = 12, N_c = 3.
 #pragma once
 #include "bril_dirs.h"
 #include "internal.h"

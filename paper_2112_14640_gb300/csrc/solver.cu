@@ -19,7 +19,7 @@
 // an unconverged run (CgScalars) and the host reads the run's norms once, at
 // its end.  BiCGstab reads them once per iteration.  (8^4, D_S, N_v = 3, FP32:
 // 76 us per iteration with three reductions' second stages, two coefficient
-// kernels and a host read in each, 28 us now; 16^3x32, D_W, N_v = 4: 0.34 and
+// kernels and a host read in each, 30 us now; 16^3x32, D_W, N_v = 4: 0.34 and
 // 0.20 ms, where the site-inner order counts too.)
 #include <math.h>
 #include <string.h>
@@ -949,7 +949,7 @@ static int reliable_solve(const dirac_op *op, const void *b, void *x, double m0,
     const auto t16 = std::chrono::steady_clock::now();
     TRY(cg_reliable(op, lo, rhs, x, m0, prm->tol, prm->maxit, delta, co, &lan, s, adaptive ? 2 : 30));
     int iters = co.iters, updates = co.recomputes;
-    if (half) {   // cg_reliable reads the residual norms on the host every iteration: the wall time is the GPU's
+    if (half) {   // cg_reliable waits for its last run and refresh: the wall time is the GPU's
         st->iters_16bit = co.iters;
         st->seconds_16bit = std::chrono::duration<double>(std::chrono::steady_clock::now() - t16).count();
     }

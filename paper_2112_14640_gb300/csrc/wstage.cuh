@@ -42,8 +42,11 @@ inline size_t smem_bytes(int T, int nchunk) {
 // with few threads per site: FP32, N_c = 3, 18x10x14x14, read by each thread
 // and staged: D_B N_v = 3: 168 and 113 us, N_v = 2: 124 and 96, blap N_v = 3: 168
 // and 109, bsuv N_v = 3: 120 and 88; N_c = 2, N_v = 2, 31x14x15x18: 224 and 150.
-// (N_c = 3, N_v = 1 does not fit.)  FP64 is bound by its own pipe: there only
-// where four threads share a site, as the ring of fewer is too large at N_c = 3.
+// (N_c = 3, N_v = 1 does not fit.)  FP64 is bound by its own pipe and D_B gains
+// little: there only where four threads share a site, as the ring of fewer is
+// too large at N_c = 3 (ms, read by each thread and staged: 16^4, N_c = 3, N_v = 4:
+// 7.37 and 7.43, 12: 21.54 and 21.64; 12^3x16, N_v = 12, N_c = 2: 4.92 and 4.88, 4: 15.91
+// and 15.42); the Laplacians in FP64 never (laplace.cuh).
 template <typename EL>
 constexpr int kMinChunks = sizeof(EL) == 8 ? 4 : 1;
 constexpr size_t kMaxSmem = 100 * 1024;
