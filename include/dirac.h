@@ -60,7 +60,7 @@ typedef enum { DIRAC_F64 = 0, DIRAC_F32 = 1, DIRAC_BF16 = 2, DIRAC_F16 = 3 } dir
 enum {
     DIRAC_OK = 0,
     DIRAC_ERR_INVALID_ARG = -1,     /* null pointer, bad enum, bad geometry */
-    DIRAC_ERR_UNSUPPORTED_NC = -2,  /* N_c outside the compiled set {1,2,3,4} */
+    DIRAC_ERR_UNSUPPORTED_NC = -2,  /* N_c outside 1..8 (1..4 with 16-bit vectors) */
     DIRAC_ERR_UNSUPPORTED_PREC = -3,
     DIRAC_ERR_ALIGNMENT = -4,       /* a vector pointer not 16-byte aligned */
     DIRAC_ERR_OOM = -5,             /* a library-owned allocation failed */
